@@ -141,14 +141,15 @@ typedef struct {
 /* Render options (36 bytes).  flags: GR_FLAG_NEE next-event estimation toward emitters
  * with power-heuristic MIS; GR_FLAG_RR Russian roulette after 3 interactions;
  * GR_FLAG_NO_RENORM keeps raw grating order weights (no renormalisation over
- * propagating orders); the default tree is the binary BVH with its child
- * boxes stored in FP16, rounded outward (32 bytes per node; used when every
- * coordinate of every scene of the call is within +-16384); GR_FLAG_FP32_NODES
- * walks the same tree with FP32 child boxes (64 bytes per node);
- * GR_FLAG_WIDE_BVH traverses the 4-wide BVH with 8-bit quantised child boxes
- * (all three give the same closest hits: a box that contains the FP32 box is
- * entered whenever the FP32 box is; the wide tree halves node visits but needs
- * more registers per thread); GR_FLAG_HERO hero-wavelength spectral MIS (Sec. 7.2):
+ * propagating orders); the default tree is the binary BVH collapsed
+ * into nodes of up to four children, with child boxes on a 16-bit grid over
+ * the scene's bounds, rounded outward (64 bytes per node; a call with a scene
+ * that has a coordinate beyond 1e12, or more than one in 16 of whose triangles
+ * is smaller than 8 steps of its grid, walks the FP32 nodes instead);
+ * GR_FLAG_FP32_NODES walks the binary tree with FP32 child boxes (64 bytes per
+ * node); GR_FLAG_WIDE_BVH traverses the 4-wide tree with 8-bit child boxes
+ * relative to each node, one ray per thread (all three give the same closest
+ * hits: a box that contains the FP32 box is entered whenever the FP32 box is); GR_FLAG_HERO hero-wavelength spectral MIS (Sec. 7.2):
  * with n_bins a multiple of 4, a path's bin is the hero of the class of bins
  * {c, c+Q, c+2Q, c+3Q} (Q = n_bins/4) and drives every sampling decision;
  * every connection to a light (escape, emitter hit, next-event estimate) is
@@ -228,8 +229,8 @@ typedef struct {
  * a BVH is built on the device: 30-bit Morton order, then agglomerative
  * clustering along that order (PLOC, window +-8, least merged surface area);
  * topology and FP32 bounds are deterministic.  The binary tree is also
- * collapsed into a 4-wide BVH with 8-bit quantised, conservatively rounded
- * child boxes.  desc arrays are host memory, read during the call only; the
+ * collapsed into 4-wide nodes, with child boxes on a 16-bit grid over the
+ * scene and with 8-bit ones relative to each node, rounded outward.  desc arrays are host memory, read during the call only; the
  * library owns the device copy until gr_scene_destroy.  The scene belongs to
  * the device current at creation and may only be rendered there.
  * Errors: GR_E_INVALID (null/negative sizes, material index out of range,

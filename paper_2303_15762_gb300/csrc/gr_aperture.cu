@@ -64,32 +64,6 @@ constexpr float kInvTwoPi = 0.159154943091895336f;
 constexpr float kNegLog2e = -1.44269504088896340736f;
 constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer (|x| < 2^22)
 
-// ---- packed FP32 pairs (one 64-bit register pair, sm_100 and later)
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
 // Hardware approximations with subnormal results and arguments as zero: the
 // forms without .ftz spend three more instructions per exponential on results
 // below 2^-126, which no sum of these terms can show.

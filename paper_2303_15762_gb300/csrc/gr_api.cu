@@ -258,10 +258,9 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
   const size_t o_etri = take(sizeof(float4) * etris.size());
   const size_t o_keys = take(sizeof(unsigned long long) * (size_t)n);
   const size_t o_wide = take(sizeof(uint4) * 4 * (size_t)std::max(n - 1, 1));
-  // FP16 nodes only when every coordinate is within +-16384 (finite boxes)
-  bool half_ok = n >= 2;
-  for (size_t i = 0; half_ok && i < 9 * (size_t)n; ++i) half_ok = std::fabs(desc->verts[i]) <= 16384.0f;
-  const size_t o_half = take(half_ok ? sizeof(uint4) * 2 * (size_t)(n - 1) : 0);
+  gr::GridDesc grid = {};
+  bool grid_ok = false;
+  const size_t o_grid = take(sizeof(uint4) * 4 * (size_t)std::max(n - 1, 0));
   int n_wide = 0;
   cudaError_t e = cudaMallocAsync(&S->mem, off, st);
   if (e != cudaSuccess) {
@@ -288,10 +287,9 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
       e = gr::build_lbvh(verts_d, tmat_in, n, (float4*)(b + o_tri), (int*)(b + o_tmat), (float*)(b + o_nodes),
                          (unsigned long long*)(b + o_keys), st);
       if (e != cudaSuccess) break;
-      e = gr::build_wide((const float*)(b + o_nodes), (const float4*)(b + o_tri), n, (uint4*)(b + o_wide), &n_wide, st);
+      e = gr::build_wide((const float*)(b + o_nodes), (const float4*)(b + o_tri), n, (uint4*)(b + o_wide),
+                         (uint4*)(b + o_grid), &grid, &grid_ok, &n_wide, st);
       if (e != cudaSuccess) break;
-      if (half_ok && (e = gr::build_half((const float*)(b + o_nodes), n, (uint4*)(b + o_half), st)) != cudaSuccess)
-        break;
     }
     // host arrays are pageable: make sure every copy has consumed them
     e = cudaStreamSynchronize(st);
@@ -313,7 +311,11 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
   D.tri_mat = (const int*)(b + o_tmat);
   D.nodes = (const float4*)(b + o_nodes);
   D.wnodes = (const uint4*)(b + o_wide);
-  D.hnodes = half_ok ? (const uint4*)(b + o_half) : nullptr;
+  D.gnodes = grid_ok ? (const uint4*)(b + o_grid) : nullptr;
+  for (int a = 0; a < 3; ++a) {
+    D.grid_lo[a] = grid.lo[a];
+    D.grid_step[a] = grid.step[a];
+  }
   D.n_wide = n_wide;
   D.pad_w = 0;
   D.mats = (const gr_material*)(b + o_mats);

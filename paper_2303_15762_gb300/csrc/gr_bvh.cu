@@ -16,6 +16,9 @@
 // precision), ties go to the lower index and node indices come from prefix
 // sums, so the result is deterministic and reproducible bit for bit by a CPU
 // build of the same algorithm.
+#include <algorithm>
+#include <cmath>
+
 #include "gr_build.h"
 
 namespace gr {
@@ -451,12 +454,79 @@ __device__ __forceinline__ float half_area(const BoxF& b) {
   return dx * dy + dy * dz + dz * dx;
 }
 
+// The 16-bit grid of a scene: its bounds in 65535 steps per axis.  It serves
+// unless a coordinate is not finite or beyond 1e12, or it is so coarse against
+// the triangles (more than one in 16 smaller than 8 steps) that their boxes
+// would swell; the renders of such a scene walk the FP32 nodes.
+struct GridState {
+  int lo[3], hi[3];  // bounds as ordered integers
+  int bad, small;    // coordinates out of range; triangles smaller than 8 steps
+  GridDesc g;
+};
+__device__ __forceinline__ int ordered(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unordered(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
+
+__global__ void k_grid_init(GridState* G) {
+  if (threadIdx.x < 3) {
+    G->lo[threadIdx.x] = 0x7fffffff;
+    G->hi[threadIdx.x] = (int)0x80000000;
+  }
+  if (threadIdx.x == 0) G->bad = G->small = 0;
+}
+__global__ void __launch_bounds__(256) k_grid_bounds(const float4* __restrict__ tri, int n, GridState* G) {
+  int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {(int)0x80000000, (int)0x80000000, (int)0x80000000};
+  bool bad = false;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n; i += gridDim.x * blockDim.x) {
+    const float4 v = tri[i];
+    const float c[3] = {v.x, v.y, v.z};
+    for (int a = 0; a < 3; ++a) {
+      bad = bad || !(fabsf(c[a]) <= 1e12f);
+      lo[a] = min(lo[a], ordered(c[a]));
+      hi[a] = max(hi[a], ordered(c[a]));
+    }
+  }
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
+    hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
+  }
+  bad = __any_sync(0xffffffffu, bad);
+  if ((threadIdx.x & 31) == 0) {
+    for (int a = 0; a < 3; ++a) {
+      atomicMin(&G->lo[a], lo[a]);
+      atomicMax(&G->hi[a], hi[a]);
+    }
+    if (bad) G->bad = 1;
+  }
+}
+__global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ tri, int n, GridState* G) {
+  GridDesc g;
+  float widest = 0.0f;
+  for (int a = 0; a < 3; ++a) {
+    g.lo[a] = unordered(G->lo[a]);
+    g.step[a] = fmaxf((float)(((double)unordered(G->hi[a]) - (double)g.lo[a]) / 65535.0 * (1.0 + 1e-6)), 1e-25f);
+    widest = fmaxf(widest, g.step[a]);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) G->g = g;
+  int small = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const BoxF b = leaf_box(tri, i);
+    small += fmaxf(fmaxf(b.hi[0] - b.lo[0], b.hi[1] - b.lo[1]), b.hi[2] - b.lo[2]) < 8.0f * widest;
+  }
+  small = __reduce_add_sync(0xffffffffu, small);
+  if ((threadIdx.x & 31) == 0 && small) atomicAdd(&G->small, small);
+}
+
 // One level of the top-down collapse: frontier item (binary node, wide index).
 __global__ void k_collapse(const float* __restrict__ nodes, const float* __restrict__ nbox,
                            const float4* __restrict__ tri, const int2* __restrict__ front, int n_front,
-                           int2* __restrict__ next, int* __restrict__ counters, uint4* __restrict__ wn) {
+                           int2* __restrict__ next, int* __restrict__ counters, uint4* __restrict__ wn,
+                           const GridState* __restrict__ G, uint4* __restrict__ gn) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_front) return;
+  const GridDesc g = G->g;
   const int bnode = front[t].x, widx = front[t].y;
   int ch[4];
   int cnt = 2;
@@ -549,121 +619,59 @@ __global__ void k_collapse(const float* __restrict__ nodes, const float* __restr
   d.y = (unsigned)refs[3];
   d.z = 0u;
   d.w = 0u;
+  for (int c = 0; c < 4; ++c) {
+    unsigned w[3];
+    for (int k = 0; k < 3; ++k) {
+      w[k] = 0xffffu;  // empty: an inverted box
+      if (c < cnt) {
+        const double lo = floor(((double)cb[c].lo[k] - (double)g.lo[k]) / (double)g.step[k]);
+        const double hi = ceil(((double)cb[c].hi[k] - (double)g.lo[k]) / (double)g.step[k]);
+        w[k] = (unsigned)fmin(fmax(lo, 0.0), 65535.0) | ((unsigned)fmin(fmax(hi, 0.0), 65535.0) << 16);
+      }
+    }
+    gn[4 * (size_t)widx + c] = make_uint4(w[0], w[1], w[2], c < cnt ? (unsigned)refs[c] : 0x80000000u);
+  }
   wn[4 * widx] = a;
   wn[4 * widx + 1] = b;
   wn[4 * widx + 2] = c4;
   wn[4 * widx + 3] = d;
 }
 
-// 32-byte binary nodes: the two child boxes of node i in FP16, each lower
-// bound rounded toward -inf and each upper bound toward +inf (so the FP16 box
-// contains the FP32 one; values beyond the FP16 range become +-inf or the
-// largest finite value on the safe side), then the two child references.
-// Halves: [l.lo.x l.lo.y][l.lo.z l.hi.x][l.hi.y l.hi.z][r.lo.x r.lo.y]
-// [r.lo.z r.hi.x][r.hi.y r.hi.z], low half of each word first.  Node i is
-// stored at position pos[i] and its internal child references are renumbered
-// the same way (leaf references are triangle slots and stay).
-__global__ void k_half_nodes(const float* __restrict__ nodes, int n, const int* __restrict__ pos,
-                             uint4* __restrict__ hn) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n - 1) return;
-  const float* N = nodes + 16 * (size_t)i;
-  unsigned short h[12];
-  for (int c = 0; c < 2; ++c)
-    for (int a = 0; a < 3; ++a) {
-      h[6 * c + a] = __half_as_ushort(__float2half_rd(N[6 * c + a]));
-      h[6 * c + 3 + a] = __half_as_ushort(__float2half_ru(N[6 * c + 3 + a]));
-    }
-  uint4 q0, q1;
-  q0.x = (unsigned)h[0] | ((unsigned)h[1] << 16);
-  q0.y = (unsigned)h[2] | ((unsigned)h[3] << 16);
-  q0.z = (unsigned)h[4] | ((unsigned)h[5] << 16);
-  q0.w = (unsigned)h[6] | ((unsigned)h[7] << 16);
-  q1.x = (unsigned)h[8] | ((unsigned)h[9] << 16);
-  q1.y = (unsigned)h[10] | ((unsigned)h[11] << 16);
-  const int l = __float_as_int(N[12]), r = __float_as_int(N[13]);
-  q1.z = (unsigned)(l >= 0 ? pos[l] : l);
-  q1.w = (unsigned)(r >= 0 ? pos[r] : r);
-  const size_t d = (size_t)pos[i];
-  hn[2 * d] = q0;
-  hn[2 * d + 1] = q1;
-}
-
 }  // namespace
 
-// FP16 copy of the binary nodes (n >= 2 leaves): hn holds (n - 1) x 32 bytes,
-// in depth-first order from the root (left child first), so that a node and
-// its left internal child are neighbours in memory and a subtree occupies one
-// contiguous range: a traversal's consecutive node fetches then often fall in
-// a cache line already read.  The order is computed on the host from the
-// nodes' child references (8 bytes per node copied back), before the
-// conversion kernel writes each node at its new position.  The tree, its
-// boxes and its closest hits are those of the FP32 nodes.
-cudaError_t build_half(const float* nodes, int n, uint4* hn, cudaStream_t st) {
-  if (n < 2) return cudaSuccess;
-  const int m = n - 1;
-  std::vector<int2> refs((size_t)m);
-  cudaError_t e = cudaMemcpy2DAsync(refs.data(), sizeof(int2), nodes + 12, 16 * sizeof(float), sizeof(int2), (size_t)m,
-                                    cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return e;
-  std::vector<int> pos((size_t)m, -1), stack;
-  stack.reserve(128);
-  stack.push_back(0);
-  int next = 0;
-  while (!stack.empty()) {
-    const int x = stack.back();
-    stack.pop_back();
-    // a malformed tree (a node reached twice, an index out of range) keeps
-    // the identity order; the traversal's own bounds then report it
-    if (x < 0 || x >= m || pos[(size_t)x] >= 0 || next >= m) {
-      next = -1;
-      break;
-    }
-    pos[(size_t)x] = next++;
-    const int2 c = refs[(size_t)x];
-    if (c.y >= 0) stack.push_back(c.y);
-    if (c.x >= 0) stack.push_back(c.x);
-  }
-  if (next != m)
-    for (int i = 0; i < m; ++i) pos[(size_t)i] = i;
-  int* pos_d = nullptr;
-  e = cudaMallocAsync(&pos_d, sizeof(int) * (size_t)m, st);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(pos_d, pos.data(), sizeof(int) * (size_t)m, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) {
-    k_half_nodes<<<(m + 255) / 256, 256, 0, st>>>(nodes, n, pos_d, hn);
-    e = cudaGetLastError();
-  }
-  // the host order must outlive its copy
-  const cudaError_t e2 = cudaStreamSynchronize(st);
-  cudaFreeAsync(pos_d, st);
-  return e != cudaSuccess ? e : e2;
-}
-
 // Collapse the binary LBVH (n >= 2 leaves) into 4-wide quantised nodes.  wn
-// must hold (n - 1) nodes (an upper bound); *n_wide receives the count.
-cudaError_t build_wide(const float* nodes, const float4* tri, int n, uint4* wn, int* n_wide, cudaStream_t st) {
+// and gn must hold (n - 1) nodes (an upper bound); *n_wide receives the count,
+// *grid the grid of gn's boxes and *grid_ok whether it serves the scene.
+cudaError_t build_wide(const float* nodes, const float4* tri, int n, uint4* wn, uint4* gn, GridDesc* grid,
+                       bool* grid_ok, int* n_wide, cudaStream_t st) {
   *n_wide = 0;
+  *grid_ok = false;
   if (n < 2) return cudaSuccess;
   float* nbox = nullptr;
   int2 *fa = nullptr, *fb = nullptr;
   int* ctr = nullptr;
   cudaError_t e = cudaSuccess;
   int h_ctr[2];
+  GridState* G = nullptr;
+  GridState h_grid;
   int n_front = 1;
   int2 root = make_int2(0, 0);
   if ((e = cudaMallocAsync(&nbox, sizeof(float) * 6 * (size_t)(n - 1), st)) != cudaSuccess) goto out;
   if ((e = cudaMallocAsync(&fa, sizeof(int2) * (size_t)n, st)) != cudaSuccess) goto out;
   if ((e = cudaMallocAsync(&fb, sizeof(int2) * (size_t)n, st)) != cudaSuccess) goto out;
   if ((e = cudaMallocAsync(&ctr, sizeof(int) * 2, st)) != cudaSuccess) goto out;
+  if ((e = cudaMallocAsync(&G, sizeof(GridState), st)) != cudaSuccess) goto out;
+  k_grid_init<<<1, 32, 0, st>>>(G);
+  k_grid_bounds<<<std::min((3 * n + 255) / 256, 1024), 256, 0, st>>>(tri, n, G);
+  k_grid_steps<<<std::min((n + 255) / 256, 1024), 256, 0, st>>>(tri, n, G);
+  if ((e = cudaMemcpyAsync(&h_grid, G, sizeof h_grid, cudaMemcpyDeviceToHost, st)) != cudaSuccess) goto out;
   k_node_boxes<<<(n - 1 + 255) / 256, 256, 0, st>>>(nodes, n, nbox);
   if ((e = cudaMemcpyAsync(fa, &root, sizeof root, cudaMemcpyHostToDevice, st)) != cudaSuccess) goto out;
   h_ctr[0] = 1;  // wide node 0 is the root
   h_ctr[1] = 0;
   if ((e = cudaMemcpyAsync(ctr, h_ctr, sizeof h_ctr, cudaMemcpyHostToDevice, st)) != cudaSuccess) goto out;
   for (int level = 0; level < 4 * 64 && n_front > 0; ++level) {
-    k_collapse<<<(n_front + 127) / 128, 128, 0, st>>>(nodes, nbox, tri, fa, n_front, fb, ctr, wn);
+    k_collapse<<<(n_front + 127) / 128, 128, 0, st>>>(nodes, nbox, tri, fa, n_front, fb, ctr, wn, G, gn);
     if ((e = cudaMemcpyAsync(h_ctr, ctr, sizeof h_ctr, cudaMemcpyDeviceToHost, st)) != cudaSuccess) goto out;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) goto out;
     n_front = h_ctr[1];
@@ -674,8 +682,11 @@ cudaError_t build_wide(const float* nodes, const float4* tri, int n, uint4* wn, 
     fb = t;
   }
   *n_wide = h_ctr[0];
+  *grid = h_grid.g;
+  *grid_ok = !h_grid.bad && (long long)h_grid.small * 16 <= n;
   e = cudaGetLastError();
 out:
+  if (G) cudaFreeAsync(G, st);
   if (nbox) cudaFreeAsync(nbox, st);
   if (fa) cudaFreeAsync(fa, st);
   if (fb) cudaFreeAsync(fb, st);

@@ -21,10 +21,14 @@ constexpr float kGCont = 50.0f;
 // Largest grating order magnitude kept in the order tables.
 constexpr int kMaxOrder = 40;
 constexpr int kStackDepth = 64;
+// the 4-wide walk pushes up to three children per two binary levels
+constexpr int kGridStackDepth = 96;
 // BVH layouts a traversal can walk: the binary tree with FP32 child boxes (64
-// bytes per node), the same tree with FP16 child boxes rounded outward (32
-// bytes per node, the default), or the 4-wide tree with 8-bit child boxes.
-enum Tree { kTreeF32 = 0, kTreeWide = 1, kTreeHalf = 2 };
+// bytes per node), its collapse into nodes of up to four children with child
+// boxes on a 16-bit grid over the scene's bounds, rounded outward (64 bytes
+// per node, the default), or the same 4-wide tree with 8-bit child boxes
+// relative to each node.
+enum Tree { kTreeF32 = 0, kTreeWide = 1, kTreeGrid = 2 };
 
 // Random-number uses at a path vertex (word 2 of the Philox counter is
 // (segment << 4) | call).
@@ -52,8 +56,11 @@ struct DevScene {
   const int* tri_mat;        // [n] material of leaf slot i
   const float4* nodes;       // [n-1][4] internal nodes (child boxes + child refs)
   const uint4* wnodes;       // [n_wide][4] 4-wide quantised nodes (root = 0)
-  const uint4* hnodes;       // [n-1][2] the binary nodes with FP16 child boxes rounded outward (32 bytes),
-                             // or null when the scene's coordinates exceed the FP16 range
+  const uint4* gnodes;       // [n_wide][4] the 4-wide nodes with child boxes on the 16-bit grid, one uint4 per
+                             // child: x, y, z bounds (lo | hi << 16) and the child reference; null when the
+                             // grid is too coarse for the scene's triangles
+  float grid_lo[3];          // the grid: coordinate = grid_lo + q * grid_step, q in [0, 65535]
+  float grid_step[3];
   int n_wide;
   int pad_w;
   const gr_material* mats;   // [n_mats]
@@ -130,6 +137,35 @@ __device__ __forceinline__ void onb_d(d3 n, d3& e1, d3& e2) {
   e1 = d3{1.0 + sign * n.x * n.x * a, sign * b, -sign * n.x};
   e2 = d3{b, sign + n.y * n.y * a, -n.y};
 }
+
+// ------------------------------------------------------------------ packed FP32
+// Pairs of FP32 values in one 64-bit register pair (sm_100 and later): each
+// half is rounded as the scalar operation rounds it.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
 
 // ------------------------------------------------------------------ Philox4x32-10
 // Salmon et al., SC'11: 10 rounds; multipliers 0xD2511F53 / 0xCD9E8D57, key
@@ -294,6 +330,40 @@ __device__ __forceinline__ float box_entry(const RayPre& r, float3 lo, float3 hi
   return tn <= tf ? tn : -1.0f;
 }
 
+// A ray on the grid of a scene's 16-bit child boxes.  A grid coordinate q
+// enters the slab test as the float v = 1 + q 2^-23, which one byte permute
+// makes from the node's word (0x3f80 above the 16 bits), so the distance to a
+// plane is the one FMA t = v s + b with s = 2^23 step / d and b = (lo - o) / d
+// - s.  Near planes get b - pad, far planes b + pad: forming b rounds by up to
+// half a grid step over |d| (|b| is about 2^23 steps), and the reciprocal, the
+// products and the distance itself by less than 12 x 2^-24 of |lo - o| / |d|
+// and of the grid's extent (2^16 steps) over |d|; pad covers their sum, so no
+// box the exact ray enters is missed.  The bytes of the near plane are chosen by the sign of d
+// (0x7610: the word's low half, the lower bound; 0x7632: its high half).
+// Components of d below 1e-18 count as +-1e-18, which keeps every value finite
+// (the pad is then far beyond any scene).
+struct GridAxis {
+  f32x2 s;       // (s, s)
+  f32x2 b;       // (near b, far b)
+  unsigned sel;  // permute of the near plane; the far plane's is sel ^ 0x22
+};
+__device__ __forceinline__ GridAxis grid_axis(float o, float d, float lo, float step) {
+  const float inv = __fdividef(1.0f, fabsf(d) < 1e-18f ? copysignf(1e-18f, d) : d);
+  const float rel = lo - o;
+  const float s = inv * (step * 8388608.0f);
+  const float pad = fabsf(inv) * fmaf(fabsf(rel), 9.5367432e-7f, 0.75f * step);
+  GridAxis g;
+  g.s = dup2(s);
+  g.b = pack2((rel * inv - pad) - s, (rel * inv + pad) - s);
+  g.sel = inv < 0.0f ? 0x7632u : 0x7610u;
+  return g;
+}
+// (near, far) distances of one child's bounds on one axis (word: lo | hi << 16).
+__device__ __forceinline__ void grid_slab(const GridAxis& g, unsigned word, float& tn, float& tf) {
+  const unsigned n = __byte_perm(word, 0x3f800000u, g.sel), f = __byte_perm(word, 0x3f800000u, g.sel ^ 0x22u);
+  unpack2(fma2(pack2(__uint_as_float(n), __uint_as_float(f)), g.s, g.b), tn, tf);
+}
+
 struct Hit {
   float t;
   int slot;  // leaf slot (BVH order) or -1
@@ -307,6 +377,7 @@ struct Hit {
 // steps are scheduled, so neither does the result.
 struct BinTrav {
   RayPre r;
+  GridAxis gx, gy, gz;  // the ray on the scene's grid (kTreeGrid only)
   float t;       // closest accepted distance so far (+inf: none)
   int slot;      // leaf slot of that hit, or -1
   int best_id;   // its original triangle id (ties go to the lower id)
@@ -331,8 +402,10 @@ __device__ __forceinline__ void bin_leaf(const float4* __restrict__ tri, BinTrav
 }
 
 // Starts a traversal; returns true if it is already complete (0 or 1 triangles).
-__device__ __forceinline__ bool bin_begin(int n_tris, const float4* __restrict__ tri, BinTrav& s, float3 o, float3 d,
-                                          int exclude, int* refined, int* tests) {
+template <int TREE>
+__device__ __forceinline__ bool bin_begin(const DevScene& S, BinTrav& s, float3 o, float3 d, int exclude, int* refined,
+                                          int* tests) {
+  const int n_tris = S.n_tris;
   s.t = __int_as_float(0x7f800000);
   s.slot = -1;
   s.best_id = 0x7fffffff;
@@ -345,22 +418,18 @@ __device__ __forceinline__ bool bin_begin(int n_tris, const float4* __restrict__
   if (n_tris == 0) return true;
   s.r = ray_pre(o, d);
   if (n_tris == 1) {
-    bin_leaf(tri, s, 0, refined, tests);
+    bin_leaf(S.tri, s, 0, refined, tests);
     return true;
+  }
+  if (TREE == kTreeGrid) {
+    s.gx = grid_axis(o.x, d.x, S.grid_lo[0], S.grid_step[0]);
+    s.gy = grid_axis(o.y, d.y, S.grid_lo[1], S.grid_step[1]);
+    s.gz = grid_axis(o.z, d.z, S.grid_lo[2], S.grid_step[2]);
   }
   return false;
 }
 
-// Two FP16 values packed in a 32-bit word (low half first), as floats.
-__device__ __forceinline__ float2 half2_bits_to_float2(unsigned w) {
-  __half2_raw r;
-  r.x = (unsigned short)(w & 0xffffu);
-  r.y = (unsigned short)(w >> 16);
-  return __half22float2(__half2(r));
-}
-
-// One node visit (HALF: the 32-byte FP16 node array, else the 64-byte FP32
-// one); returns true when the traversal is complete.  Leaf
+// One visit of an FP32 node; returns true when the traversal is complete.  Leaf
 // children whose boxes the ray enters go to leaf(slot), which tests them at
 // once or queues them: the closest hit is the least (t, original id) over the
 // tested triangles whatever the order of the tests, and a test only ever
@@ -368,7 +437,7 @@ __device__ __forceinline__ float2 half2_bits_to_float2(unsigned w) {
 // bound trips, 1 if the stack would overflow (the traversal then drops the
 // farther child).  `stack` holds kStackDepth entries, kept outside BinTrav so
 // that the ray state stays in registers.
-template <bool HALF, class LeafFn>
+template <class LeafFn>
 __device__ __forceinline__ bool bin_step(const void* __restrict__ nodes, BinTrav& s, int* stack, int* visits,
                                          int* err, LeafFn&& leaf) {
   if (--s.guard < 0) {
@@ -378,27 +447,17 @@ __device__ __forceinline__ bool bin_step(const void* __restrict__ nodes, BinTrav
   ++*visits;
   float tl, tr;
   int lref, rref;
-  if (HALF) {
-    // 32-byte node: halves [l.lo.x l.lo.y][l.lo.z l.hi.x][l.hi.y l.hi.z]
-    // [r.lo.x r.lo.y][r.lo.z r.hi.x][r.hi.y r.hi.z], then lref, rref; the
-    // boxes contain the FP32 ones, so a box the FP32 tree enters is entered
-    const uint4* N = (const uint4*)nodes + 2 * s.node;
-    const uint4 q0 = __ldg(N), q1 = __ldg(N + 1);
-    const float2 a = half2_bits_to_float2(q0.x), b = half2_bits_to_float2(q0.y), c = half2_bits_to_float2(q0.z);
-    const float2 d = half2_bits_to_float2(q0.w), e = half2_bits_to_float2(q1.x), f = half2_bits_to_float2(q1.y);
-    lref = (int)q1.z;
-    rref = (int)q1.w;
-    tl = box_entry(s.r, f3(a.x, a.y, b.x), f3(b.y, c.x, c.y), s.t);
-    tr = box_entry(s.r, f3(d.x, d.y, e.x), f3(e.y, f.x, f.y), s.t);
-  } else {
+  bool hl, hr;
+  {
     const float4* N = (const float4*)nodes + 4 * s.node;
     const float4 n0 = __ldg(N), n1 = __ldg(N + 1), n2 = __ldg(N + 2), n3 = __ldg(N + 3);
     lref = __float_as_int(n3.x);
     rref = __float_as_int(n3.y);
     tl = box_entry(s.r, f3(n0.x, n0.y, n0.z), f3(n0.w, n1.x, n1.y), s.t);
     tr = box_entry(s.r, f3(n1.z, n1.w, n2.x), f3(n2.y, n2.z, n2.w), s.t);
+    hl = tl >= 0.0f;
+    hr = tr >= 0.0f;
   }
-  bool hl = tl >= 0.0f, hr = tr >= 0.0f;
   // leaves go to `leaf`; internal children are descended/pushed
   if (hl && lref < 0) {
     leaf(lref & 0x7fffffff);
@@ -431,30 +490,59 @@ __device__ __forceinline__ bool bin_step(const void* __restrict__ nodes, BinTrav
   return false;
 }
 
-// Closest hit along (o, d) with t > kTMin, skipping leaf slot `exclude`;
-// equal distances resolve to the lower original triangle id.  Stack-based
-// traversal of the binary BVH, nearer child first.  *err is set if the stack
-// would overflow (the traversal then stops early).
-template <bool HALF = false>
-__device__ __forceinline__ Hit closest_hit(const DevScene& S, float3 o, float3 d, int exclude, int* refined,
-                                           int* visits, int* tests, int* err) {
-  BinTrav s;
-  int stack[kStackDepth];
-  if (!bin_begin(S.n_tris, S.tri, s, o, d, exclude, refined, tests)) {
-    const float4* tri = S.tri;
-    auto test_now = [&](int leaf) { bin_leaf(tri, s, leaf, refined, tests); };
-    const void* nodes = HALF ? (const void*)S.hnodes : (const void*)S.nodes;
-    while (!bin_step<HALF>(nodes, s, stack, visits, err, test_now)) {
-    }
+// One visit of a 4-wide grid node (same contract as bin_step).  The boxes
+// contain the FP32 ones, so a triangle that the FP32 tree tests is tested.
+// The nearest internal child is walked next (entry distances as ordered
+// integers with the child's index in the two low bits), the others are pushed
+// in child order: a sorting network over all four saves 0.6% of the visits and
+// costs 1% of the time.  An empty child has an inverted box, and leaf slot 0
+// as its reference in case a degenerate grid lets a ray in all the same.
+template <class LeafFn>
+__device__ __forceinline__ bool grid_step(const uint4* __restrict__ nodes, BinTrav& s, int* stack, int* visits,
+                                          int* err, LeafFn&& leaf) {
+  if (--s.guard < 0) {
+    if (err) *err = 2;
+    return true;
   }
-  Hit h;
-  h.t = s.t;
-  h.slot = s.slot;
-  return h;
+  ++*visits;
+  const uint4* N = nodes + 4 * (size_t)(unsigned)s.node;
+  uint4 c[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c[k] = __ldg(N + k);
+  constexpr unsigned kNone = 0xffffffffu;
+  unsigned key[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float nx, ny, nz, fx, fy, fz;
+    grid_slab(s.gx, c[k].x, nx, fx);
+    grid_slab(s.gy, c[k].y, ny, fy);
+    grid_slab(s.gz, c[k].z, nz, fz);
+    const float tn = fmaxf(fmaxf(nx, ny), fmaxf(nz, 0.0f));
+    const bool hit = tn <= fminf(fminf(fx, fy), fminf(fz, s.t));
+    const int ref = (int)c[k].w;
+    if (hit && ref < 0) leaf(ref & 0x7fffffff);
+    key[k] = hit && ref >= 0 ? (__float_as_uint(tn) & ~3u) | (unsigned)k : kNone;
+  }
+  const unsigned near = min(min(key[0], key[1]), min(key[2], key[3]));
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (key[k] != kNone && key[k] != near) {
+      if (s.sp < kGridStackDepth) stack[s.sp++] = (int)c[k].w;
+      else if (err) *err = 1;
+    }
+  if (near != kNone) {
+    const unsigned a = near & 1u ? c[1].w : c[0].w, b = near & 1u ? c[3].w : c[2].w;
+    s.node = (int)(near & 2u ? b : a);
+    return false;
+  }
+  if (s.sp == 0) return true;
+  s.node = stack[--s.sp];
+  return false;
 }
 
-// Closest hit through the 4-wide quantised BVH: same contract as closest_hit
-// (t > kTMin, skip `exclude`, ties to the lower original id).  A node decodes
+// Closest hit along (o, d) through the 4-wide quantised BVH: t > kTMin, leaf
+// slot `exclude` skipped, equal distances resolve to the lower original
+// triangle id (as the binary tree's walk).  A node decodes
 // its child slabs as t = q * (2^e / d) + (P - o) / d, one FMA per bound; the
 // far distance is widened by 8 ulps and the near one narrowed, so rounding
 // can only add visits.

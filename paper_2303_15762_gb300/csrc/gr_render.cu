@@ -625,22 +625,41 @@ __global__ void __launch_bounds__(256) k_regen(RenderParams p) {
 #ifndef GR_TRACE_STEPS
 #define GR_TRACE_STEPS 6
 #endif
-// Closest hits for a queue of rays on the binary tree, one warp keeping its 32
+#ifndef GR_GRID_STEPS
+#define GR_GRID_STEPS 6
+#endif
+// leaves a lane of the 4-wide walk can hold
+#ifndef GR_GRID_LEAVES
+#define GR_GRID_LEAVES 6
+#endif
+constexpr int kGridLeaves = GR_GRID_LEAVES;
+// Closest hits for a queue of rays on the binary tree (FP32 nodes) or on its
+// 4-wide grid nodes (the default), one warp keeping its 32
 // lanes busy across rays.  Warps claim the queue in groups of 32 entries from
 // `cursor`; a lane whose ray has finished stays idle until GR_TRACE_REFILL
 // lanes are idle (or every lane is), then the idle lanes take the next
 // entries together, so ray set-up runs once per batch rather than once per
 // lane, the warp no longer waits for the slowest ray of a fixed group of 32,
 // and all warps advance through the queue together (neighbouring rays share
-// BVH nodes in L1).  Leaf triangles are queued per lane (up to 3; a lane
-// holding 2 stops walking) and tested in warp-wide passes once GR_LEAF_BATCH
+// BVH nodes in L1).  Leaf triangles are queued per lane (up to 3 in registers,
+// a lane holding 2 stops walking; 4-wide: up to kGridLeaves in shared memory,
+// a lane without room for four more stops) and tested in warp-wide passes once GR_LEAF_BATCH
 // lanes hold some, or GR_LEAF_BLOCKED lanes are stopped, or no lane can walk:
-// one test then serves many lanes instead of two or three.  The hit equals
-// closest_hit's (the least (t, id) over the triangles whose boxes the ray
-// enters); only the counts of visits and tests differ.
+// one test then serves many lanes instead of two or three.  The hit is the
+// least (t, id) over the triangles whose boxes the ray enters, whatever the
+// tree and the schedule; only the counts of visits and tests differ.
+// What bounds it: the chain of dependent node fetches (long-scoreboard stalls
+// of 4 warps per issue) beside 58% busy ALUs at 17 of 32 lanes.  The 4-wide
+// grid nodes halve the chain: 13.2 visits per ray instead of 26.0, and 20%
+// fewer instructions; k_trace on 129M rays of a 512^2 x 256 spp render of 91k
+// triangles went from 38.6 to 32.1 ms (binary nodes with FP16 boxes before;
+// the same binary nodes on the grid: 37.8).  kGridLeaves 4 / 5 / 8: 34.4 /
+// 33.6 / 33.6 ms against 32.9 at 6; 2 / 3 / 4 visits between two looks at the
+// schedule: 35.4 / 34.0 / 32.9 ms against 32.5 at 6; 6 or 8 blocks per SM:
+// 34.3 / 37.1 ms against 34.0 at 7.
 //   entry(e) -> slot of queue entry e; ray(slot, o, d, exclude) gives the
 //   ray and returns its scene; done(slot, hit) consumes a finished ray.
-template <bool HALF, class Entry, class Ray, class Done>
+template <int TREE, class Entry, class Ray, class Done>
 __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cursor, Entry&& entry, Ray&& ray,
                                            Done&& done, int& refined, int& visits, int& tests, int& err) {
   const int lane = threadIdx.x & 31;
@@ -648,7 +667,7 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
   BinTrav s;
   s.t = 0.0f;
   s.slot = -1;
-  int stack[kStackDepth];
+  int stack[TREE == kTreeGrid ? kGridStackDepth : kStackDepth];
   const void* nodes = nullptr;
   const float4* tri = nullptr;
   int out = -1;
@@ -656,9 +675,15 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
   bool walking = false;  // ... whose node walk has not ended
   int np = 0, pl0 = 0, pl1 = 0, pl2 = 0;  // queued leaves (at most 3)
   int exclude = -1;                        // the ray's s.exclude, kept for the queueing test
+  // the lane's queued leaves: three registers, or kGridLeaves words of shared
+  // memory for the 4-wide nodes, which can add four at a visit
+  constexpr bool GRID = TREE == kTreeGrid;
+  __shared__ int s_leaf[GRID ? kGridLeaves : 1][GRID ? GR_TRACE_BLOCK : 1];
+  constexpr int kFull = GRID ? kGridLeaves - 3 : 2;  // a lane holding as many stops walking
   auto queue_leaf = [&](int leaf) {
     if (leaf == exclude) return;
-    if (np == 0) pl0 = leaf;
+    if (GRID) s_leaf[np][threadIdx.x] = leaf;
+    else if (np == 0) pl0 = leaf;
     else if (np == 1) pl1 = leaf;
     else pl2 = leaf;
     ++np;
@@ -674,6 +699,7 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
   const int group = n > GR_TRACE_BIG_QUEUE ? 64 : 32;
   int base = 0, left = 0;
   bool more = true;  // unclaimed groups may remain
+  constexpr int kSteps = GRID ? GR_GRID_STEPS : GR_TRACE_STEPS;
   for (;;) {
     const unsigned idle = __ballot_sync(0xffffffffu, !live);
     if (idle == 0xffffffffu && !more && left == 0) break;
@@ -704,12 +730,12 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
         int x = -1;
         float3 o, d;
         const DevScene& S = ray(slot, o, d, x);
-        nodes = HALF ? (const void*)S.hnodes : (const void*)S.nodes;
+        nodes = TREE == kTreeGrid ? (const void*)S.gnodes : (const void*)S.nodes;
         tri = S.tri;
         out = slot;
         np = 0;
         exclude = x;
-        live = walking = !bin_begin(S.n_tris, tri, s, o, d, x, &refined, &tests);
+        live = walking = !bin_begin<TREE>(S, s, o, d, x, &refined, &tests);
         if (!live) {
           live = true;
           finish();
@@ -717,29 +743,37 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
       }
     }
     // leaf pass: the queued triangles of many lanes are tested together
-    const bool blocked = live && (np >= 2 || (!walking && np > 0));
+    const bool blocked = live && (np >= kFull || (!walking && np > 0));
     const unsigned pend = __ballot_sync(0xffffffffu, live && np > 0);
     const unsigned blk = __ballot_sync(0xffffffffu, blocked);
-    const unsigned can_walk = __ballot_sync(0xffffffffu, live && walking && np < 2);
+    const unsigned can_walk = __ballot_sync(0xffffffffu, live && walking && np < kFull);
     if (pend && (__popc(pend) >= GR_LEAF_BATCH || __popc(blk) >= GR_LEAF_BLOCKED || can_walk == 0)) {
       if (live && np > 0) {
-        bin_leaf(tri, s, pl0, &refined, &tests);
-        if (np > 1) bin_leaf(tri, s, pl1, &refined, &tests);
-        if (np > 2) bin_leaf(tri, s, pl2, &refined, &tests);
+        if (GRID) {
+#pragma unroll 1
+          for (int q = 0; q < np; ++q) bin_leaf(tri, s, s_leaf[q][threadIdx.x], &refined, &tests);
+        } else {
+          bin_leaf(tri, s, pl0, &refined, &tests);
+          if (np > 1) bin_leaf(tri, s, pl1, &refined, &tests);
+          if (np > 2) bin_leaf(tri, s, pl2, &refined, &tests);
+        }
         np = 0;
         if (!walking) finish();
       }
     }
 #pragma unroll 1
-    for (int k = 0; k < GR_TRACE_STEPS && live && walking && np < 2; ++k) {
-      walking = !bin_step<HALF>(nodes, s, stack, &visits, &err, queue_leaf);
+    for (int k = 0; k < kSteps && live && walking && np < kFull; ++k) {
+      if (GRID)
+        walking = !grid_step((const uint4*)nodes, s, stack, &visits, &err, queue_leaf);
+      else
+        walking = !bin_step(nodes, s, stack, &visits, &err, queue_leaf);
       if (!walking && np == 0) finish();
     }
   }
 }
 
 // Closest hits of the trace queue and of the next-event rays the previous
-// k_shade requested, in one launch: the binary tree (FP32 or FP16 child boxes)
+// k_shade requested, in one launch: the binary or 4-wide grid nodes
 // through lane_trace, the 4-wide tree one ray per thread per pass.  Entries
 // [0, ns) are the next-event rays (origin: the vertex, direction: the sampled
 // emitter direction; their hits go to shh), then the trace queue, which holds
@@ -772,7 +806,7 @@ __global__ void __launch_bounds__(TREE == kTreeWide ? 256 : GR_TRACE_BLOCK, TREE
       (es & kShadowEntry ? P.shh : P.hit)[slot] = make_float2(h.t, __int_as_float(h.slot));
     }
   } else {
-    lane_trace<TREE == kTreeHalf>(
+    lane_trace<TREE>(
         p, n, &p.ctr->trace_next, [&](int e) { return trace_entry(p, e, ns, front); },
         [&](int es, float3& o, float3& d, int& exclude) -> const DevScene& {
           const int slot = es & ~kShadowEntry;
@@ -2259,8 +2293,8 @@ cudaError_t launch_iteration(const RenderParams& p, int tree, int grid_regen, in
                              int grid_shadow, int block, size_t smem, cudaStream_t st, cudaEvent_t* ev) {
   if (tree == kTreeWide)
     return launch_iteration_t<NS, TT, kTreeWide>(p, grid_regen, grid_trace, grid_shade, grid_shadow, block, smem, st, ev);
-  if (tree == kTreeHalf)
-    return launch_iteration_t<NS, TT, kTreeHalf>(p, grid_regen, grid_trace, grid_shade, grid_shadow, block, smem, st, ev);
+  if (tree == kTreeGrid)
+    return launch_iteration_t<NS, TT, kTreeGrid>(p, grid_regen, grid_trace, grid_shade, grid_shadow, block, smem, st, ev);
   return launch_iteration_t<NS, TT, kTreeF32>(p, grid_regen, grid_trace, grid_shade, grid_shadow, block, smem, st, ev);
 }
 
@@ -2285,18 +2319,17 @@ const void* shade_kernel(int ns, int dtype, int mode) {
 }
 const void* trace_kernel(int tree) {
   return tree == kTreeWide ? (const void*)k_trace<kTreeWide>
-                           : tree == kTreeHalf ? (const void*)k_trace<kTreeHalf> : (const void*)k_trace<kTreeF32>;
+                           : tree == kTreeGrid ? (const void*)k_trace<kTreeGrid> : (const void*)k_trace<kTreeF32>;
 }
-// The tree a render walks: the 4-wide one on request, else the FP16 binary
-// nodes unless FP32 nodes are requested or a scene has no FP16 nodes (its
-// coordinates exceed the FP16 range; scenes of fewer than 2 triangles need no
-// nodes).
+// The tree a render walks: the 8-bit 4-wide one on request, else the 4-wide
+// nodes on the 16-bit grid unless FP32 nodes are requested or a scene has no
+// grid nodes (GridState; scenes of fewer than 2 triangles need no nodes).
 int pick_tree(int flags, gr_scene* const* scenes, int n_scenes) {
   if (flags & GR_FLAG_WIDE_BVH) return kTreeWide;
   if (flags & GR_FLAG_FP32_NODES) return kTreeF32;
   for (int i = 0; i < n_scenes; ++i)
-    if (scenes[i]->n_tris >= 2 && !scenes[i]->dev.hnodes) return kTreeF32;
-  return kTreeHalf;
+    if (scenes[i]->n_tris >= 2 && !scenes[i]->dev.gnodes) return kTreeF32;
+  return kTreeGrid;
 }
 const void* regen_kernel(int ns, bool hero) {
   if (ns == 1) return hero ? (const void*)k_regen<1, true> : (const void*)k_regen<1, false>;
