@@ -284,11 +284,9 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
     if ((e = cudaMemcpyAsync(b + o_eom, emitter_of_mat.data(), sizeof(int) * emitter_of_mat.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
     if (!etris.empty() && (e = cudaMemcpyAsync(b + o_etri, etris.data(), sizeof(float4) * etris.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
     if (n > 0) {
-      e = gr::build_lbvh(verts_d, tmat_in, n, (float4*)(b + o_tri), (int*)(b + o_tmat), (float*)(b + o_nodes),
-                         (unsigned long long*)(b + o_keys), st);
-      if (e != cudaSuccess) break;
-      e = gr::build_wide((const float*)(b + o_nodes), (const float4*)(b + o_tri), n, (uint4*)(b + o_wide),
-                         (uint4*)(b + o_grid), &grid, &grid_ok, &n_wide, st);
+      e = gr::build_trees(verts_d, tmat_in, n, (float4*)(b + o_tri), (int*)(b + o_tmat), (float*)(b + o_nodes),
+                          (unsigned long long*)(b + o_keys), (uint4*)(b + o_wide), (uint4*)(b + o_grid), &grid,
+                          &grid_ok, &n_wide, st);
       if (e != cudaSuccess) break;
     }
     // host arrays are pageable: make sure every copy has consumed them

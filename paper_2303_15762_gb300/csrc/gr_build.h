@@ -11,14 +11,13 @@
 
 namespace gr {
 
-cudaError_t build_lbvh(const float* verts, const int* tri_mat, int n, float4* tri, int* tmat, float* nodes,
-                       unsigned long long* keys_out, cudaStream_t st);
 // The 16-bit grid of the default nodes' child boxes: coordinate = lo + q step.
 struct GridDesc {
   float lo[3], step[3];
 };
-cudaError_t build_wide(const float* nodes, const float4* tri, int n, uint4* wn, uint4* gn, GridDesc* grid,
-                       bool* grid_ok, int* n_wide, cudaStream_t st);
+cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* tri, int* tmat, float* nodes,
+                        unsigned long long* keys_out, uint4* wn, uint4* gn, GridDesc* grid, bool* grid_ok,
+                        int* n_wide, cudaStream_t st);
 
 // Largest slot pool (the trace launch tags next-event entries with bit 30 of
 // the slot index).

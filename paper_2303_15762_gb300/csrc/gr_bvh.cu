@@ -33,47 +33,90 @@ __device__ __forceinline__ unsigned expand_bits(unsigned v) {
   return v;
 }
 
-__global__ void k_centroids(const float* __restrict__ verts, int n, float4* __restrict__ cen) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float* v = verts + 9 * i;
-  float cx = __fdiv_rn(__fadd_rn(__fadd_rn(v[0], v[3]), v[6]), 3.0f);
-  float cy = __fdiv_rn(__fadd_rn(__fadd_rn(v[1], v[4]), v[7]), 3.0f);
-  float cz = __fdiv_rn(__fadd_rn(__fadd_rn(v[2], v[5]), v[8]), 3.0f);
-  cen[i] = make_float4(cx, cy, cz, 0.0f);
+// Order-preserving integers of floats (for atomic minima and maxima; -0 sorts
+// below +0, and both decode to themselves).
+__device__ __forceinline__ int ordered(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unordered(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
+
+// What the build's kernels pass on through device memory, so that the host
+// waits for none of them until the tree is done.
+constexpr int kMaxLevels = 256;
+struct BuildState {
+  int clo[3], chi[3];   // centroid bounds as ordered integers
+  int lo[3], hi[3];     // vertex bounds as ordered integers
+  int bad, small;       // coordinates out of the grid's range; triangles smaller than 8 grid steps
+  GridDesc g;
+  int m[2], created[2]; // clusters left and nodes created, by parity of the round
+  int level_first[kMaxLevels + 1], level_count[kMaxLevels + 1];  // wide nodes of each level
+};
+__global__ void k_build_init(BuildState* B, int n) {
+  const int t = threadIdx.x;
+  if (t < 3) {
+    B->clo[t] = B->lo[t] = 0x7fffffff;
+    B->chi[t] = B->hi[t] = (int)0x80000000;
+  }
+  if (t == 0) {
+    B->bad = B->small = 0;
+    B->m[0] = n;
+    B->created[0] = 0;
+  }
+  for (int l = t; l <= kMaxLevels; l += blockDim.x) {
+    B->level_first[l] = 0;
+    B->level_count[l] = l == 0 ? 1 : 0;
+  }
 }
 
-// One block reduces the centroid bounds (exact min/max).
-__global__ void k_bounds(const float4* __restrict__ cen, int n, float* __restrict__ out6) {
-  __shared__ float s[6][1024];
-  float lo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, hi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    float4 c = cen[i];
-    lo[0] = fminf(lo[0], c.x);
-    lo[1] = fminf(lo[1], c.y);
-    lo[2] = fminf(lo[2], c.z);
-    hi[0] = fmaxf(hi[0], c.x);
-    hi[1] = fmaxf(hi[1], c.y);
-    hi[2] = fmaxf(hi[2], c.z);
-  }
+// Centroids, and the bounds of centroids and vertices (exact min/max: a warp
+// reduction and one atomic per warp).
+__global__ void __launch_bounds__(256) k_centroids(const float* __restrict__ verts, int n, float4* __restrict__ cen,
+                                                   BuildState* B) {
+  int clo[3], chi[3], lo[3], hi[3];
   for (int a = 0; a < 3; ++a) {
-    s[a][threadIdx.x] = lo[a];
-    s[3 + a][threadIdx.x] = hi[a];
+    clo[a] = lo[a] = 0x7fffffff;
+    chi[a] = hi[a] = (int)0x80000000;
   }
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      for (int a = 0; a < 3; ++a) {
-        s[a][threadIdx.x] = fminf(s[a][threadIdx.x], s[a][threadIdx.x + w]);
-        s[3 + a][threadIdx.x] = fmaxf(s[3 + a][threadIdx.x], s[3 + a][threadIdx.x + w]);
+  bool bad = false;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const float* v = verts + 9 * (size_t)i;
+    float c[3];
+    for (int a = 0; a < 3; ++a) {
+      c[a] = __fdiv_rn(__fadd_rn(__fadd_rn(v[a], v[3 + a]), v[6 + a]), 3.0f);
+      // a centroid that is not a number leaves the bounds as they are
+      if (c[a] == c[a]) {
+        clo[a] = min(clo[a], ordered(c[a]));
+        chi[a] = max(chi[a], ordered(c[a]));
+      }
+      for (int k = 0; k < 3; ++k) {
+        const float x = v[3 * k + a];
+        bad = bad || !(fabsf(x) <= 1e12f);
+        lo[a] = min(lo[a], ordered(x));
+        hi[a] = max(hi[a], ordered(x));
       }
     }
-    __syncthreads();
+    cen[i] = make_float4(c[0], c[1], c[2], 0.0f);
   }
-  if (threadIdx.x < 6) out6[threadIdx.x] = s[threadIdx.x][0];
+  bad = __any_sync(0xffffffffu, bad);
+  for (int a = 0; a < 3; ++a) {
+    clo[a] = __reduce_min_sync(0xffffffffu, clo[a]);
+    chi[a] = __reduce_max_sync(0xffffffffu, chi[a]);
+    lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
+    hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    for (int a = 0; a < 3; ++a) {
+      atomicMin(&B->clo[a], clo[a]);
+      atomicMax(&B->chi[a], chi[a]);
+      atomicMin(&B->lo[a], lo[a]);
+      atomicMax(&B->hi[a], hi[a]);
+    }
+    if (bad) B->bad = 1;
+  }
 }
 
-__global__ void k_morton(const float4* __restrict__ cen, int n, int n_pad, const float* __restrict__ b6,
+__global__ void k_morton(const float4* __restrict__ cen, int n, int n_pad, const BuildState* __restrict__ B,
                          unsigned long long* __restrict__ keys) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_pad) return;
@@ -85,8 +128,9 @@ __global__ void k_morton(const float4* __restrict__ cen, int n, int n_pad, const
   float cc[3] = {c.x, c.y, c.z};
   unsigned q[3];
   for (int a = 0; a < 3; ++a) {
-    float ext = __fsub_rn(b6[3 + a], b6[a]);
-    float t = ext > 0.0f ? __fdiv_rn(__fsub_rn(cc[a], b6[a]), ext) : 0.0f;
+    const float lo = unordered(B->clo[a]);
+    float ext = __fsub_rn(unordered(B->chi[a]), lo);
+    float t = ext > 0.0f ? __fdiv_rn(__fsub_rn(cc[a], lo), ext) : 0.0f;
     int qi = (int)__fmul_rn(t, 1024.0f);
     qi = qi < 0 ? 0 : (qi > 1023 ? 1023 : qi);
     q[a] = (unsigned)qi;
@@ -201,54 +245,110 @@ __global__ void k_leaf_clusters(const float4* __restrict__ tri, int n, float* __
   C[i] = i | 0x80000000;
 }
 
-// Nearest neighbour of every cluster within the window (least merged area,
-// ties to the lower index).
-__global__ void k_ploc_nn(const float* __restrict__ B, int m, int* __restrict__ N) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const Box6 bi = load_box(B, i);
+// One cluster's nearest neighbour within the window: least merged area, ties
+// to the lower index.  box(j) gives cluster j's box.
+template <class BoxFn>
+__device__ __forceinline__ int nearest(int i, int m, BoxFn&& box) {
+  const Box6 bi = box(i);
   int best = -1;
   float ba = 3.4e38f;
-  const int j0 = i - kPlocRadius < 0 ? 0 : i - kPlocRadius;
-  const int j1 = i + kPlocRadius > m - 1 ? m - 1 : i + kPlocRadius;
+  const int j0 = max(i - kPlocRadius, 0), j1 = min(i + kPlocRadius, m - 1);
   for (int j = j0; j <= j1; ++j) {
     if (j == i) continue;
-    const float a = half_area_rn(box_union(bi, load_box(B, j)));
+    const float a = half_area_rn(box_union(bi, box(j)));
     if (a < ba || (a == ba && j < best)) {
       ba = a;
       best = j;
     }
   }
-  N[i] = best;
+  return best;
 }
 
-// Flags: bit 0 = i merges with its (higher-index) mutual neighbour, bit 1 =
-// i survives compaction (it is not the higher index of a mutual pair).
-__global__ void k_ploc_flags(const int* __restrict__ N, int m, int2* __restrict__ F) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const int j = N[i];
-  const bool mutual = j >= 0 && N[j] == i;
-  F[i] = make_int2((mutual && i < j) ? 1 : 0, (mutual && j < i) ? 0 : 1);
+__device__ __forceinline__ void write_node(float* __restrict__ Nd, const Box6& a, const Box6& b, int ca, int cb) {
+  float4* q = (float4*)Nd;
+  q[0] = make_float4(a.lo[0], a.lo[1], a.lo[2], a.hi[0]);
+  q[1] = make_float4(a.hi[1], a.hi[2], b.lo[0], b.lo[1]);
+  q[2] = make_float4(b.lo[2], b.hi[0], b.hi[1], b.hi[2]);
+  q[3] = make_float4(__int_as_float(ca), __int_as_float(cb), 0.0f, 0.0f);
 }
 
-// Exclusive scan of the flag pairs with one block (m up to a few million):
-// each thread sums a contiguous chunk, the block scans the partial sums,
-// then each thread writes its chunk's prefixes.  totals = (merges, survivors).
-__global__ void k_scan_pairs(const int2* __restrict__ F, int m, int2* __restrict__ S, int2* __restrict__ totals) {
+// A round of the clustering over many blocks is three launches; the cluster
+// count is read from device memory, so the host enqueues rounds without
+// waiting (blocks beyond the count return, and rounds that start with at most
+// kTail clusters do nothing).  Until every round was counted on the host the
+// build of 91k triangles waited ~30 times and scanned its flags with one block:
+// scene creation 3.3 -> 2.1 ms (1.01M triangles: 23.9 -> 5.6).
+constexpr int kTile = 256, kTail = 1024;
+// levels of the collapse enqueued at a time (a scene that takes more waits once more per batch)
+constexpr int kLevelBatch = 18;
+
+// Nearest neighbours of a tile (and of the 8 clusters on either side, whose
+// choice decides who is mutual), the pairs that merge, and the tile's counts.
+// P[i] = j when i merges with the higher-index j, -1 when i stays, -2 when it
+// is merged away.
+__global__ void __launch_bounds__(kTile) k_ploc_pairs(const float* __restrict__ B, const BuildState* __restrict__ S,
+                                                      int parity, int* __restrict__ P, int2* __restrict__ sums) {
+  const int m = S->m[parity], start = blockIdx.x * kTile;
+  if (m <= kTail || start >= m) return;
+  constexpr int H = 2 * kPlocRadius;
+  __shared__ float s_box[(kTile + 2 * H) * 6];
+  __shared__ int s_nn[kTile + 2 * kPlocRadius];
+  __shared__ int2 s_cnt[kTile / 32];
+  const int first = max(start - H, 0), last = min(start + kTile + H, m);
+  for (int i = threadIdx.x; i < (last - first) * 6; i += kTile) s_box[i] = B[6 * (size_t)first + i];
+  __syncthreads();
+  auto box = [&](int j) { return load_box(s_box, j - first); };
+  for (int q = threadIdx.x; q < kTile + 2 * kPlocRadius; q += kTile) {
+    const int i = start - kPlocRadius + q;
+    s_nn[q] = i >= 0 && i < m ? nearest(i, m, box) : -1;
+  }
+  __syncthreads();
+  const int i = start + threadIdx.x;
+  bool merges = false, stays = false;
+  if (i < m) {
+    const int j = s_nn[threadIdx.x + kPlocRadius];
+    const bool mutual = j >= 0 && s_nn[j - start + kPlocRadius] == i;
+    merges = mutual && i < j;
+    stays = !(mutual && j < i);
+    P[i] = merges ? j : stays ? -1 : -2;
+  }
+  const unsigned a = __ballot_sync(0xffffffffu, merges), c = __ballot_sync(0xffffffffu, stays);
+  if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = make_int2(__popc(a), __popc(c));
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int2 t = make_int2(0, 0);
+    for (int w = 0; w < kTile / 32; ++w) {
+      t.x += s_cnt[w].x;
+      t.y += s_cnt[w].y;
+    }
+    sums[blockIdx.x] = t;
+  }
+}
+
+// Exclusive prefix of the tiles' counts (one block: a contiguous chunk per
+// thread, a scan of the partial sums, the chunk's prefixes) and the next
+// round's cluster and node counts.
+__global__ void __launch_bounds__(1024) k_ploc_scan(int2* __restrict__ sums, BuildState* S, int parity) {
+  const int m = S->m[parity], created = S->created[parity], t = threadIdx.x;
+  if (m <= kTail) {
+    if (t == 0) {
+      S->m[parity ^ 1] = m;
+      S->created[parity ^ 1] = created;
+    }
+    return;
+  }
   __shared__ int2 part[1024];
-  const int t = threadIdx.x;
-  const int chunk = (m + blockDim.x - 1) / blockDim.x;
-  const int b = t * chunk, e = min(m, b + chunk);
+  const int tiles = (m + kTile - 1) / kTile, chunk = (tiles + 1023) / 1024;
+  const int b = min(t * chunk, tiles), e = min(b + chunk, tiles);
   int2 acc = make_int2(0, 0);
   for (int i = b; i < e; ++i) {
-    acc.x += F[i].x;
-    acc.y += F[i].y;
+    acc.x += sums[i].x;
+    acc.y += sums[i].y;
   }
   part[t] = acc;
   __syncthreads();
-  for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-    int2 v = t >= off ? part[t - off] : make_int2(0, 0);
+  for (int off = 1; off < 1024; off <<= 1) {
+    const int2 v = t >= off ? part[t - off] : make_int2(0, 0);
     __syncthreads();
     part[t].x += v.x;
     part[t].y += v.y;
@@ -256,44 +356,126 @@ __global__ void k_scan_pairs(const int2* __restrict__ F, int m, int2* __restrict
   }
   int2 run = t > 0 ? part[t - 1] : make_int2(0, 0);
   for (int i = b; i < e; ++i) {
-    S[i] = run;
-    run.x += F[i].x;
-    run.y += F[i].y;
+    const int2 v = sums[i];
+    sums[i] = run;
+    run.x += v.x;
+    run.y += v.y;
   }
-  if (t == (int)blockDim.x - 1) *totals = part[t];
+  if (t == 1023) {
+    S->m[parity ^ 1] = part[1023].y;
+    S->created[parity ^ 1] = created + part[1023].x;
+  }
 }
 
-// Merge mutual pairs into new nodes (index (n-2) - creation order, so the
-// root, created last, is node 0) and compact the clusters in order.
-__global__ void k_ploc_apply(const float* __restrict__ B, const int* __restrict__ C, const int* __restrict__ N,
-                             const int2* __restrict__ F, const int2* __restrict__ S, int m, int n, int created,
-                             float* __restrict__ B2, int* __restrict__ C2, float* __restrict__ nodes) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const int2 f = F[i];
-  if (!f.y) return;
-  const int2 pos = S[i];
-  const Box6 bi = load_box(B, i);
-  if (f.x) {
-    const int j = N[i];
-    const Box6 bj = load_box(B, j);
-    const int x = (n - 2) - (created + pos.x);
-    float* Nd = nodes + 16 * x;
-    for (int k = 0; k < 3; ++k) {
-      Nd[k] = bi.lo[k];
-      Nd[3 + k] = bi.hi[k];
-      Nd[6 + k] = bj.lo[k];
-      Nd[9 + k] = bj.hi[k];
+// Merge the pairs into new nodes (index (n-2) - creation order, so the root,
+// created last, is node 0) and compact the clusters in order.
+__global__ void __launch_bounds__(kTile) k_ploc_merge(const float* __restrict__ B, const int* __restrict__ C,
+                                                      const int* __restrict__ P, const int2* __restrict__ sums,
+                                                      const BuildState* __restrict__ S, int parity, int n,
+                                                      float* __restrict__ B2, int* __restrict__ C2,
+                                                      float* __restrict__ nodes) {
+  const int m = S->m[parity], start = blockIdx.x * kTile;
+  if (start >= m) return;
+  const int i = start + threadIdx.x;
+  if (m <= kTail) {  // the round is over before it began: the clusters move to the other buffer
+    if (i < m) {
+      store_box(B2, i, load_box(B, i));
+      C2[i] = C[i];
     }
-    Nd[12] = __int_as_float(C[i]);
-    Nd[13] = __int_as_float(C[j]);
-    Nd[14] = 0.0f;
-    Nd[15] = 0.0f;
+    return;
+  }
+  __shared__ int2 s_cnt[kTile / 32];
+  const int j = i < m ? P[i] : -2;
+  const unsigned a = __ballot_sync(0xffffffffu, j >= 0), c = __ballot_sync(0xffffffffu, j >= -1);
+  if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = make_int2(__popc(a), __popc(c));
+  __syncthreads();
+  if (j == -2) return;
+  const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
+  int2 pos = sums[blockIdx.x];
+  for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) {
+    pos.x += s_cnt[w].x;
+    pos.y += s_cnt[w].y;
+  }
+  pos.x += __popc(a & below);
+  pos.y += __popc(c & below);
+  const Box6 bi = load_box(B, i);
+  if (j >= 0) {
+    const Box6 bj = load_box(B, j);
+    const int x = (n - 2) - (S->created[parity] + pos.x);
+    write_node(nodes + 16 * (size_t)x, bi, bj, C[i], C[j]);
     store_box(B2, pos.y, box_union(bi, bj));
     C2[pos.y] = x;
   } else {
     store_box(B2, pos.y, bi);
     C2[pos.y] = C[i];
+  }
+}
+
+// The last rounds, from at most kTail clusters to one, in one block's shared
+// memory (one cluster per thread).
+__global__ void __launch_bounds__(kTail) k_ploc_tail(const float* __restrict__ B, const int* __restrict__ C,
+                                                     BuildState* S, int parity, int n, float* __restrict__ nodes) {
+  int m = S->m[parity], created = S->created[parity];
+  if (m > kTail) return;
+  __shared__ float s_box[kTail * 6];
+  __shared__ int s_id[kTail], s_nn[kTail];
+  __shared__ int2 s_cnt[kTail / 32];
+  const int i = threadIdx.x, warp = i >> 5;
+  const unsigned below = (1u << (i & 31)) - 1u;
+  for (int q = i; q < 6 * m; q += kTail) s_box[q] = B[q];
+  if (i < m) s_id[i] = C[i];
+  __syncthreads();
+  auto box = [&](int j) { return load_box(s_box, j); };
+  // a round with more than one cluster merges at least one pair: at most kTail - 1 rounds
+  for (int round = 0; m > 1 && round < kTail; ++round) {
+    if (i < m) s_nn[i] = nearest(i, m, box);
+    __syncthreads();
+    const int j = i < m ? s_nn[i] : -1;
+    const bool mutual = j >= 0 && s_nn[j] == i;
+    const bool merges = mutual && i < j, stays = i < m && !(mutual && j < i);
+    const unsigned a = __ballot_sync(0xffffffffu, merges), c = __ballot_sync(0xffffffffu, stays);
+    if ((i & 31) == 0) s_cnt[warp] = make_int2(__popc(a), __popc(c));
+    Box6 bi, bj;
+    int id = 0, idj = 0;
+    if (stays) {
+      bi = box(i);
+      id = s_id[i];
+    }
+    if (merges) {
+      bj = box(j);
+      idj = s_id[j];
+    }
+    __syncthreads();
+    int2 pos = make_int2(0, 0), tot = make_int2(0, 0);
+    const int warps = (m + 31) >> 5;
+    for (int w = 0; w < warps; ++w) {
+      const int2 v = s_cnt[w];
+      if (w < warp) {
+        pos.x += v.x;
+        pos.y += v.y;
+      }
+      tot.x += v.x;
+      tot.y += v.y;
+    }
+    pos.x += __popc(a & below);
+    pos.y += __popc(c & below);
+    if (merges) {
+      const int x = (n - 2) - (created + pos.x);
+      write_node(nodes + 16 * (size_t)x, bi, bj, id, idj);
+      bi = box_union(bi, bj);
+      id = x;
+    }
+    if (stays) {
+      store_box(s_box, pos.y, bi);
+      s_id[pos.y] = id;
+    }
+    created += tot.x;
+    m = tot.y;
+    __syncthreads();
+  }
+  if (i == 0) {
+    S->m[parity] = m;
+    S->created[parity] = created;
   }
 }
 
@@ -312,84 +494,6 @@ inline cudaError_t launch_sort(unsigned long long* keys, int n_pad, cudaStream_t
 }
 
 }  // namespace
-
-// Build the BVH of `n` triangles (device arrays verts [n][9], tri_mat [n]).
-// Outputs (device, caller-allocated): tri [n][3] float4, tmat [n], nodes
-// [(n-1)][16] floats, keys [n_pad].  Scratch is allocated here and freed
-// before return (stream-ordered).
-cudaError_t build_lbvh(const float* verts, const int* tri_mat, int n, float4* tri, int* tmat, float* nodes,
-                       unsigned long long* keys_out, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  int n_pad = 2048;
-  while (n_pad < n) n_pad <<= 1;
-  float4* cen = nullptr;
-  float* b6 = nullptr;
-  unsigned long long* keys = nullptr;
-  float* Bb = nullptr;
-  int *Cb = nullptr, *Nn = nullptr;
-  int2 *Fl = nullptr, *Sc = nullptr, *Tot = nullptr;
-  cudaError_t e = cudaSuccess;
-#define GR_TRY(x)                 \
-  do {                            \
-    e = (x);                      \
-    if (e != cudaSuccess) goto done; \
-  } while (0)
-  GR_TRY(cudaMallocAsync(&cen, sizeof(float4) * n, st));
-  GR_TRY(cudaMallocAsync(&b6, sizeof(float) * 6, st));
-  GR_TRY(cudaMallocAsync(&keys, sizeof(unsigned long long) * n_pad, st));
-  k_centroids<<<(n + 255) / 256, 256, 0, st>>>(verts, n, cen);
-  k_bounds<<<1, 1024, 0, st>>>(cen, n, b6);
-  k_morton<<<(n_pad + 255) / 256, 256, 0, st>>>(cen, n, n_pad, b6, keys);
-  GR_TRY(cudaGetLastError());
-  GR_TRY(launch_sort(keys, n_pad, st));
-  k_reorder<<<(n + 255) / 256, 256, 0, st>>>(keys, n, verts, tri_mat, tri, tmat);
-  GR_TRY(cudaGetLastError());
-  if (n > 1) {
-    GR_TRY(cudaMallocAsync(&Bb, sizeof(float) * 6 * 2 * (size_t)n, st));
-    GR_TRY(cudaMallocAsync(&Cb, sizeof(int) * 2 * (size_t)n, st));
-    GR_TRY(cudaMallocAsync(&Nn, sizeof(int) * (size_t)n, st));
-    GR_TRY(cudaMallocAsync(&Fl, sizeof(int2) * (size_t)n, st));
-    GR_TRY(cudaMallocAsync(&Sc, sizeof(int2) * (size_t)n, st));
-    GR_TRY(cudaMallocAsync(&Tot, sizeof(int2), st));
-    float* Bc = Bb;
-    float* Bn = Bb + 6 * (size_t)n;
-    int* Cc = Cb;
-    int* Cn = Cb + n;
-    k_leaf_clusters<<<(n + 255) / 256, 256, 0, st>>>(tri, n, Bc, Cc);
-    int m = n, created = 0;
-    for (int it = 0; m > 1 && it < n; ++it) {
-      const int g = (m + 255) / 256;
-      k_ploc_nn<<<g, 256, 0, st>>>(Bc, m, Nn);
-      k_ploc_flags<<<g, 256, 0, st>>>(Nn, m, Fl);
-      k_scan_pairs<<<1, 1024, 0, st>>>(Fl, m, Sc, Tot);
-      k_ploc_apply<<<g, 256, 0, st>>>(Bc, Cc, Nn, Fl, Sc, m, n, created, Bn, Cn, nodes);
-      int2 tot;
-      GR_TRY(cudaMemcpyAsync(&tot, Tot, sizeof tot, cudaMemcpyDeviceToHost, st));
-      GR_TRY(cudaStreamSynchronize(st));
-      created += tot.x;
-      m = tot.y;
-      std::swap(Bc, Bn);
-      std::swap(Cc, Cn);
-    }
-    if (m != 1 || created != n - 1) {
-      e = cudaErrorUnknown;
-      goto done;
-    }
-  }
-  if (keys_out) GR_TRY(cudaMemcpyAsync(keys_out, keys, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, st));
-done:
-  if (cen) cudaFreeAsync(cen, st);
-  if (b6) cudaFreeAsync(b6, st);
-  if (keys) cudaFreeAsync(keys, st);
-  if (Bb) cudaFreeAsync(Bb, st);
-  if (Cb) cudaFreeAsync(Cb, st);
-  if (Nn) cudaFreeAsync(Nn, st);
-  if (Fl) cudaFreeAsync(Fl, st);
-  if (Sc) cudaFreeAsync(Sc, st);
-  if (Tot) cudaFreeAsync(Tot, st);
-#undef GR_TRY
-  return e;
-}
 
 // ------------------------------------------------------------------ 4-wide quantised BVH
 // Derived from the binary LBVH: each wide node takes a binary node and expands
@@ -422,23 +526,6 @@ __device__ __forceinline__ BoxF leaf_box(const float4* tri, int slot) {
   return r;
 }
 
-// Box of every binary internal node (from its parent's child-box slots).
-__global__ void k_node_boxes(const float* __restrict__ nodes, int n, float* __restrict__ nbox) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n - 1) return;
-  const float* N = nodes + 16 * i;
-  const int l = __float_as_int(N[12]), r = __float_as_int(N[13]);
-  if (l >= 0)
-    for (int k = 0; k < 6; ++k) nbox[6 * l + k] = N[k];
-  if (r >= 0)
-    for (int k = 0; k < 6; ++k) nbox[6 * r + k] = N[6 + k];
-  if (i == 0)
-    for (int k = 0; k < 3; ++k) {
-      nbox[k] = fminf(N[k], N[6 + k]);
-      nbox[3 + k] = fmaxf(N[3 + k], N[9 + k]);
-    }
-}
-
 __device__ __forceinline__ BoxF ref_box(int ref, const float* nbox, const float4* tri) {
   if (ref < 0) return leaf_box(tri, ref & 0x7fffffff);
   BoxF b;
@@ -457,77 +544,61 @@ __device__ __forceinline__ float half_area(const BoxF& b) {
 // The 16-bit grid of a scene: its bounds in 65535 steps per axis.  It serves
 // unless a coordinate is not finite or beyond 1e12, or it is so coarse against
 // the triangles (more than one in 16 smaller than 8 steps) that their boxes
-// would swell; the renders of such a scene walk the FP32 nodes.
-struct GridState {
-  int lo[3], hi[3];  // bounds as ordered integers
-  int bad, small;    // coordinates out of range; triangles smaller than 8 steps
-  GridDesc g;
-};
-__device__ __forceinline__ int ordered(float f) {
-  const int i = __float_as_int(f);
-  return i ^ ((i >> 31) & 0x7fffffff);
-}
-__device__ __forceinline__ float unordered(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
-
-__global__ void k_grid_init(GridState* G) {
-  if (threadIdx.x < 3) {
-    G->lo[threadIdx.x] = 0x7fffffff;
-    G->hi[threadIdx.x] = (int)0x80000000;
-  }
-  if (threadIdx.x == 0) G->bad = G->small = 0;
-}
-__global__ void __launch_bounds__(256) k_grid_bounds(const float4* __restrict__ tri, int n, GridState* G) {
-  int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {(int)0x80000000, (int)0x80000000, (int)0x80000000};
-  bool bad = false;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n; i += gridDim.x * blockDim.x) {
-    const float4 v = tri[i];
-    const float c[3] = {v.x, v.y, v.z};
-    for (int a = 0; a < 3; ++a) {
-      bad = bad || !(fabsf(c[a]) <= 1e12f);
-      lo[a] = min(lo[a], ordered(c[a]));
-      hi[a] = max(hi[a], ordered(c[a]));
-    }
-  }
-  for (int a = 0; a < 3; ++a) {
-    lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
-    hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
-  }
-  bad = __any_sync(0xffffffffu, bad);
-  if ((threadIdx.x & 31) == 0) {
-    for (int a = 0; a < 3; ++a) {
-      atomicMin(&G->lo[a], lo[a]);
-      atomicMax(&G->hi[a], hi[a]);
-    }
-    if (bad) G->bad = 1;
-  }
-}
-__global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ tri, int n, GridState* G) {
+// would swell; the renders of such a scene walk the FP32 nodes.  The same
+// launch stores the box of every binary internal node (from its parent's
+// child boxes).
+__global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ tri, const float* __restrict__ nodes, int n,
+                                                    BuildState* S, int parity, float* __restrict__ nbox,
+                                                    int* __restrict__ front) {
+  if (S->m[parity] != 1) return;  // the clustering needs more rounds
   GridDesc g;
   float widest = 0.0f;
   for (int a = 0; a < 3; ++a) {
-    g.lo[a] = unordered(G->lo[a]);
-    g.step[a] = fmaxf((float)(((double)unordered(G->hi[a]) - (double)g.lo[a]) / 65535.0 * (1.0 + 1e-6)), 1e-25f);
+    g.lo[a] = unordered(S->lo[a]);
+    g.step[a] = fmaxf((float)(((double)unordered(S->hi[a]) - (double)g.lo[a]) / 65535.0 * (1.0 + 1e-6)), 1e-25f);
     widest = fmaxf(widest, g.step[a]);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) G->g = g;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    S->g = g;
+    front[0] = 0;  // wide node 0 stands for the root
+  }
   int small = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const BoxF b = leaf_box(tri, i);
     small += fmaxf(fmaxf(b.hi[0] - b.lo[0], b.hi[1] - b.lo[1]), b.hi[2] - b.lo[2]) < 8.0f * widest;
+    if (i >= n - 1) continue;
+    const float4* q = (const float4*)(nodes + 16 * (size_t)i);
+    const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
+    const float N[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
+    const int l = __float_as_int(q3.x), r = __float_as_int(q3.y);
+    if (l >= 0)
+      for (int k = 0; k < 6; ++k) nbox[6 * (size_t)l + k] = N[k];
+    if (r >= 0)
+      for (int k = 0; k < 6; ++k) nbox[6 * (size_t)r + k] = N[6 + k];
+    if (i == 0)
+      for (int k = 0; k < 3; ++k) {
+        nbox[k] = fminf(N[k], N[6 + k]);
+        nbox[3 + k] = fmaxf(N[3 + k], N[9 + k]);
+      }
   }
   small = __reduce_add_sync(0xffffffffu, small);
-  if ((threadIdx.x & 31) == 0 && small) atomicAdd(&G->small, small);
+  if ((threadIdx.x & 31) == 0 && small) atomicAdd(&S->small, small);
 }
 
-// One level of the top-down collapse: frontier item (binary node, wide index).
-__global__ void k_collapse(const float* __restrict__ nodes, const float* __restrict__ nbox,
-                           const float4* __restrict__ tri, const int2* __restrict__ front, int n_front,
-                           int2* __restrict__ next, int* __restrict__ counters, uint4* __restrict__ wn,
-                           const GridState* __restrict__ G, uint4* __restrict__ gn) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_front) return;
-  const GridDesc g = G->g;
-  const int bnode = front[t].x, widx = front[t].y;
+// One level of the top-down collapse.  front[w] is the binary node that wide
+// node w stands for; level L's nodes are [level_first[L], + level_count[L]),
+// and a node's internal children take consecutive places in the next level.
+__global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ nodes, const float* __restrict__ nbox,
+                                                  const float4* __restrict__ tri, int* __restrict__ front,
+                                                  BuildState* S, int parity, int level, uint4* __restrict__ wn,
+                                                  uint4* __restrict__ gn) {
+  if (S->m[parity] != 1) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int first = S->level_first[level], count = S->level_count[level];
+  if (t == 0) S->level_first[level + 1] = first + count;
+  if (t >= count) return;
+  const GridDesc g = S->g;
+  const int widx = first + t, bnode = front[widx];
   int ch[4];
   int cnt = 2;
   ch[0] = __float_as_int(nodes[16 * bnode + 12]);
@@ -588,14 +659,15 @@ __global__ void k_collapse(const float* __restrict__ nodes, const float* __restr
     }
   }
   int refs[4] = {-1, -1, -1, -1};
+  int inner = 0;
+  for (int c = 0; c < cnt; ++c) inner += ch[c] >= 0;
+  int w = inner ? first + count + atomicAdd(&S->level_count[level + 1], inner) : 0;
   for (int c = 0; c < cnt; ++c) {
     if (ch[c] < 0) {
       refs[c] = ch[c];
     } else {
-      const int w = atomicAdd(counters + 0, 1);
       refs[c] = w;
-      const int f = atomicAdd(counters + 1, 1);
-      next[f] = make_int2(ch[c], w);
+      front[w++] = ch[c];
     }
   }
   uint4 a, b, c4, d;
@@ -639,58 +711,98 @@ __global__ void k_collapse(const float* __restrict__ nodes, const float* __restr
 
 }  // namespace
 
-// Collapse the binary LBVH (n >= 2 leaves) into 4-wide quantised nodes.  wn
-// and gn must hold (n - 1) nodes (an upper bound); *n_wide receives the count,
-// *grid the grid of gn's boxes and *grid_ok whether it serves the scene.
-cudaError_t build_wide(const float* nodes, const float4* tri, int n, uint4* wn, uint4* gn, GridDesc* grid,
-                       bool* grid_ok, int* n_wide, cudaStream_t st) {
+// Build the trees of `n` triangles (device arrays verts [n][9], tri_mat [n]).
+// Outputs (device, caller-allocated): tri [n][3] float4, tmat [n], nodes
+// [(n-1)][16] floats, keys [n], and the 4-wide nodes wn and gn of up to n - 1
+// nodes each; on the host *n_wide (their count), *grid (the grid of gn's
+// boxes) and *grid_ok (whether it serves the scene).  One scratch allocation;
+// the host waits once, for the state the launches leave behind, and again only
+// if the clustering or the collapse takes more rounds than were enqueued.
+cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* tri, int* tmat, float* nodes,
+                        unsigned long long* keys_out, uint4* wn, uint4* gn, GridDesc* grid, bool* grid_ok,
+                        int* n_wide, cudaStream_t st) {
   *n_wide = 0;
   *grid_ok = false;
-  if (n < 2) return cudaSuccess;
-  float* nbox = nullptr;
-  int2 *fa = nullptr, *fb = nullptr;
-  int* ctr = nullptr;
-  cudaError_t e = cudaSuccess;
-  int h_ctr[2];
-  GridState* G = nullptr;
-  GridState h_grid;
-  int n_front = 1;
-  int2 root = make_int2(0, 0);
-  if ((e = cudaMallocAsync(&nbox, sizeof(float) * 6 * (size_t)(n - 1), st)) != cudaSuccess) goto out;
-  if ((e = cudaMallocAsync(&fa, sizeof(int2) * (size_t)n, st)) != cudaSuccess) goto out;
-  if ((e = cudaMallocAsync(&fb, sizeof(int2) * (size_t)n, st)) != cudaSuccess) goto out;
-  if ((e = cudaMallocAsync(&ctr, sizeof(int) * 2, st)) != cudaSuccess) goto out;
-  if ((e = cudaMallocAsync(&G, sizeof(GridState), st)) != cudaSuccess) goto out;
-  k_grid_init<<<1, 32, 0, st>>>(G);
-  k_grid_bounds<<<std::min((3 * n + 255) / 256, 1024), 256, 0, st>>>(tri, n, G);
-  k_grid_steps<<<std::min((n + 255) / 256, 1024), 256, 0, st>>>(tri, n, G);
-  if ((e = cudaMemcpyAsync(&h_grid, G, sizeof h_grid, cudaMemcpyDeviceToHost, st)) != cudaSuccess) goto out;
-  k_node_boxes<<<(n - 1 + 255) / 256, 256, 0, st>>>(nodes, n, nbox);
-  if ((e = cudaMemcpyAsync(fa, &root, sizeof root, cudaMemcpyHostToDevice, st)) != cudaSuccess) goto out;
-  h_ctr[0] = 1;  // wide node 0 is the root
-  h_ctr[1] = 0;
-  if ((e = cudaMemcpyAsync(ctr, h_ctr, sizeof h_ctr, cudaMemcpyHostToDevice, st)) != cudaSuccess) goto out;
-  for (int level = 0; level < 4 * 64 && n_front > 0; ++level) {
-    k_collapse<<<(n_front + 127) / 128, 128, 0, st>>>(nodes, nbox, tri, fa, n_front, fb, ctr, wn, G, gn);
-    if ((e = cudaMemcpyAsync(h_ctr, ctr, sizeof h_ctr, cudaMemcpyDeviceToHost, st)) != cudaSuccess) goto out;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) goto out;
-    n_front = h_ctr[1];
-    h_ctr[1] = 0;
-    if ((e = cudaMemcpyAsync(ctr + 1, &h_ctr[1], sizeof(int), cudaMemcpyHostToDevice, st)) != cudaSuccess) goto out;
-    int2* t = fa;
-    fa = fb;
-    fb = t;
-  }
-  *n_wide = h_ctr[0];
-  *grid = h_grid.g;
-  *grid_ok = !h_grid.bad && (long long)h_grid.small * 16 <= n;
-  e = cudaGetLastError();
-out:
-  if (G) cudaFreeAsync(G, st);
-  if (nbox) cudaFreeAsync(nbox, st);
-  if (fa) cudaFreeAsync(fa, st);
-  if (fb) cudaFreeAsync(fb, st);
-  if (ctr) cudaFreeAsync(ctr, st);
+  if (n <= 0) return cudaSuccess;
+  int n_pad = 2048;
+  while (n_pad < n) n_pad <<= 1;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t r = off;
+    off += (bytes + 255) / 256 * 256;
+    return r;
+  };
+  const size_t N = (size_t)n, o_state = take(sizeof(BuildState)), o_cen = take(sizeof(float4) * N);
+  const size_t o_keys = take(sizeof(unsigned long long) * (size_t)n_pad);
+  const size_t o_box = take(sizeof(float) * 6 * 2 * N), o_id = take(sizeof(int) * 2 * N), o_p = take(sizeof(int) * N);
+  const size_t o_sums = take(sizeof(int2) * (N / kTile + 1));
+  unsigned char* d = nullptr;
+  cudaError_t e = cudaMallocAsync((void**)&d, off, st);
+  if (e != cudaSuccess) return e;
+  BuildState* S = (BuildState*)(d + o_state);
+  float4* cen = (float4*)(d + o_cen);
+  unsigned long long* keys = (unsigned long long*)(d + o_keys);
+  float *Bc = (float*)(d + o_box), *Bn = Bc + 6 * N;
+  int *Cc = (int*)(d + o_id), *Cn = Cc + N, *P = (int*)(d + o_p);
+  int2* sums = (int2*)(d + o_sums);
+  BuildState h;
+  auto run = [&]() -> cudaError_t {
+    const int g256 = (n + 255) / 256;
+    cudaError_t r;
+    k_build_init<<<1, 256, 0, st>>>(S, n);
+    k_centroids<<<std::min(g256, 1024), 256, 0, st>>>(verts, n, cen, S);
+    k_morton<<<(n_pad + 255) / 256, 256, 0, st>>>(cen, n, n_pad, S, keys);
+    if ((r = launch_sort(keys, n_pad, st)) != cudaSuccess) return r;
+    k_reorder<<<g256, 256, 0, st>>>(keys, n, verts, tri_mat, tri, tmat);
+    if ((r = cudaMemcpyAsync(keys_out, keys, sizeof(unsigned long long) * N, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
+      return r;
+    if (n == 1) return cudaGetLastError();
+    k_leaf_clusters<<<g256, 256, 0, st>>>(tri, n, Bc, Cc);
+    // rounds of the many-block form: a round leaves about 0.65 of the clusters
+    int parity = 0;
+    for (long long bound = n, done = 0; done < n;) {
+      int rounds = 0;
+      for (double m = (double)bound; m > kTail; m *= 0.7) ++rounds;
+      const int tiles = (int)((bound + kTile - 1) / kTile);
+      for (int k = 0; k < rounds; ++k) {
+        k_ploc_pairs<<<tiles, kTile, 0, st>>>(Bc, S, parity, P, sums);
+        k_ploc_scan<<<1, 1024, 0, st>>>(sums, S, parity);
+        k_ploc_merge<<<tiles, kTile, 0, st>>>(Bc, Cc, P, sums, S, parity, n, Bn, Cn, nodes);
+        std::swap(Bc, Bn);
+        std::swap(Cc, Cn);
+        parity ^= 1;
+      }
+      done += rounds;
+      k_ploc_tail<<<1, kTail, 0, st>>>(Bc, Cc, S, parity, n, nodes);
+      // the collapse is enqueued with the rounds; its launches return at once
+      // if the clustering is not done, and are enqueued again after the next ones
+      float* nbox = Bc;  // the cluster boxes and ids have served
+      int* front = Cc;
+      k_grid_steps<<<std::min(g256, 1024), 256, 0, st>>>(tri, nodes, n, S, parity, nbox, front);
+      int level = 0;
+      do {
+        for (int k = 0; k < kLevelBatch && level < kMaxLevels; ++k, ++level) {
+          const double widest = level < 14 ? std::pow(4.0, level) : 3e8;
+          const int blocks = (int)((std::min(widest, (double)n) + 127) / 128);
+          k_collapse<<<blocks, 128, 0, st>>>(nodes, nbox, tri, front, S, parity, level, wn, gn);
+        }
+        if ((r = cudaMemcpyAsync(&h, S, sizeof h, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return r;
+        if ((r = cudaStreamSynchronize(st)) != cudaSuccess) return r;
+      } while (h.m[parity] == 1 && h.level_count[level] > 0 && level < kMaxLevels);
+      if (h.m[parity] == 1) {
+        if (h.created[parity] != n - 1 || h.level_count[level] > 0) return cudaErrorUnknown;
+        *n_wide = h.level_first[level];
+        *grid = h.g;
+        *grid_ok = !h.bad && (long long)h.small * 16 <= n;
+        return cudaGetLastError();
+      }
+      if (rounds == 0 || h.m[parity] >= bound) break;  // no pair merges (boxes that are not finite)
+      bound = h.m[parity];
+    }
+    return cudaErrorUnknown;
+  };
+  e = run();
+  cudaFreeAsync(d, st);
   return e;
 }
 
