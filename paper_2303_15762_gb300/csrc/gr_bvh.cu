@@ -50,6 +50,7 @@ struct BuildState {
   int bad, small;       // coordinates out of the grid's range; triangles smaller than 8 grid steps
   GridDesc g;
   int m[2], created[2]; // clusters left and nodes created, by parity of the round
+  int tiles_done;       // tiles of the round that have counted their pairs
   int level_first[kMaxLevels + 1], level_count[kMaxLevels + 1];  // wide nodes of each level
 };
 __global__ void k_build_init(BuildState* B, int n) {
@@ -59,7 +60,7 @@ __global__ void k_build_init(BuildState* B, int n) {
     B->chi[t] = B->hi[t] = (int)0x80000000;
   }
   if (t == 0) {
-    B->bad = B->small = 0;
+    B->bad = B->small = B->tiles_done = 0;
     B->m[0] = n;
     B->created[0] = 0;
   }
@@ -98,22 +99,29 @@ __global__ void __launch_bounds__(256) k_centroids(const float* __restrict__ ver
     }
     cen[i] = make_float4(c[0], c[1], c[2], 0.0f);
   }
-  bad = __any_sync(0xffffffffu, bad);
+  // one set of atomics per block
+  __shared__ int s_b[12][8];
+  __shared__ int s_bad;
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int a = 0; a < 3; ++a) {
-    clo[a] = __reduce_min_sync(0xffffffffu, clo[a]);
-    chi[a] = __reduce_max_sync(0xffffffffu, chi[a]);
-    lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
-    hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
+    const int v[4] = {__reduce_min_sync(0xffffffffu, clo[a]), __reduce_max_sync(0xffffffffu, chi[a]),
+                      __reduce_min_sync(0xffffffffu, lo[a]), __reduce_max_sync(0xffffffffu, hi[a])};
+    if (lane == 0)
+      for (int k = 0; k < 4; ++k) s_b[4 * a + k][warp] = v[k];
   }
-  if ((threadIdx.x & 31) == 0) {
-    for (int a = 0; a < 3; ++a) {
-      atomicMin(&B->clo[a], clo[a]);
-      atomicMax(&B->chi[a], chi[a]);
-      atomicMin(&B->lo[a], lo[a]);
-      atomicMax(&B->hi[a], hi[a]);
-    }
-    if (bad) B->bad = 1;
+  if (bad) s_bad = 1;
+  __syncthreads();
+  if (threadIdx.x < 12) {
+    const int a = threadIdx.x >> 2, k = threadIdx.x & 3;
+    int v = s_b[threadIdx.x][0];
+    for (int w = 1; w < 8; ++w) v = k & 1 ? max(v, s_b[threadIdx.x][w]) : min(v, s_b[threadIdx.x][w]);
+    int* at = k == 0 ? &B->clo[a] : k == 1 ? &B->chi[a] : k == 2 ? &B->lo[a] : &B->hi[a];
+    if (k & 1) atomicMax(at, v);
+    else atomicMin(at, v);
   }
+  if (threadIdx.x == 0 && s_bad) B->bad = 1;
 }
 
 __global__ void k_morton(const float4* __restrict__ cen, int n, int n_pad, const BuildState* __restrict__ B,
@@ -272,98 +280,100 @@ __device__ __forceinline__ void write_node(float* __restrict__ Nd, const Box6& a
   q[3] = make_float4(__int_as_float(ca), __int_as_float(cb), 0.0f, 0.0f);
 }
 
-// A round of the clustering over many blocks is three launches; the cluster
+// A round of the clustering over many blocks is two launches; the cluster
 // count is read from device memory, so the host enqueues rounds without
 // waiting (blocks beyond the count return, and rounds that start with at most
 // kTail clusters do nothing).  Until every round was counted on the host the
 // build of 91k triangles waited ~30 times and scanned its flags with one block:
-// scene creation 3.3 -> 2.1 ms (1.01M triangles: 23.9 -> 5.6).
+// scene creation 3.3 -> 1.24 ms (1.01M triangles: 23.9 -> 3.8).
 constexpr int kTile = 256, kTail = 1024;
+constexpr int kPairThreads = kTile + 32;  // the tile and the clusters on either side, a thread each
 // levels of the collapse enqueued at a time (a scene that takes more waits once more per batch)
 constexpr int kLevelBatch = 18;
 
 // Nearest neighbours of a tile (and of the 8 clusters on either side, whose
 // choice decides who is mutual), the pairs that merge, and the tile's counts.
 // P[i] = j when i merges with the higher-index j, -1 when i stays, -2 when it
-// is merged away.
-__global__ void __launch_bounds__(kTile) k_ploc_pairs(const float* __restrict__ B, const BuildState* __restrict__ S,
-                                                      int parity, int* __restrict__ P, int2* __restrict__ sums) {
-  const int m = S->m[parity], start = blockIdx.x * kTile;
-  if (m <= kTail || start >= m) return;
-  constexpr int H = 2 * kPlocRadius;
-  __shared__ float s_box[(kTile + 2 * H) * 6];
-  __shared__ int s_nn[kTile + 2 * kPlocRadius];
-  __shared__ int2 s_cnt[kTile / 32];
-  const int first = max(start - H, 0), last = min(start + kTile + H, m);
-  for (int i = threadIdx.x; i < (last - first) * 6; i += kTile) s_box[i] = B[6 * (size_t)first + i];
-  __syncthreads();
-  auto box = [&](int j) { return load_box(s_box, j - first); };
-  for (int q = threadIdx.x; q < kTile + 2 * kPlocRadius; q += kTile) {
-    const int i = start - kPlocRadius + q;
-    s_nn[q] = i >= 0 && i < m ? nearest(i, m, box) : -1;
-  }
-  __syncthreads();
-  const int i = start + threadIdx.x;
-  bool merges = false, stays = false;
-  if (i < m) {
-    const int j = s_nn[threadIdx.x + kPlocRadius];
-    const bool mutual = j >= 0 && s_nn[j - start + kPlocRadius] == i;
-    merges = mutual && i < j;
-    stays = !(mutual && j < i);
-    P[i] = merges ? j : stays ? -1 : -2;
-  }
-  const unsigned a = __ballot_sync(0xffffffffu, merges), c = __ballot_sync(0xffffffffu, stays);
-  if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = make_int2(__popc(a), __popc(c));
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int2 t = make_int2(0, 0);
-    for (int w = 0; w < kTile / 32; ++w) {
-      t.x += s_cnt[w].x;
-      t.y += s_cnt[w].y;
-    }
-    sums[blockIdx.x] = t;
-  }
-}
-
-// Exclusive prefix of the tiles' counts (one block: a contiguous chunk per
-// thread, a scan of the partial sums, the chunk's prefixes) and the next
-// round's cluster and node counts.
-__global__ void __launch_bounds__(1024) k_ploc_scan(int2* __restrict__ sums, BuildState* S, int parity) {
-  const int m = S->m[parity], created = S->created[parity], t = threadIdx.x;
+// is merged away.  The last tile to finish turns the counts into their
+// exclusive prefixes and sets the next round's cluster and node counts.
+__global__ void __launch_bounds__(kPairThreads) k_ploc_pairs(const float* __restrict__ B, BuildState* S, int parity,
+                                                             int* __restrict__ P, int2* sums) {
+  const int m = S->m[parity], created = S->created[parity], start = blockIdx.x * kTile, t = threadIdx.x;
   if (m <= kTail) {
-    if (t == 0) {
+    if (blockIdx.x == 0 && t == 0) {
       S->m[parity ^ 1] = m;
       S->created[parity ^ 1] = created;
     }
     return;
   }
-  __shared__ int2 part[1024];
-  const int tiles = (m + kTile - 1) / kTile, chunk = (tiles + 1023) / 1024;
-  const int b = min(t * chunk, tiles), e = min(b + chunk, tiles);
-  int2 acc = make_int2(0, 0);
-  for (int i = b; i < e; ++i) {
-    acc.x += sums[i].x;
-    acc.y += sums[i].y;
-  }
-  part[t] = acc;
+  if (start >= m) return;
+  constexpr int H = 2 * kPlocRadius;
+  __shared__ float s_box[(kTile + 2 * H) * 6];
+  __shared__ int s_nn[kTile + H];
+  __shared__ int2 s_cnt[kPairThreads / 32];
+  __shared__ int2 s_part[kPairThreads];
+  __shared__ int s_last;
+  const int first = max(start - H, 0), last = min(start + kTile + H, m);
+  for (int i = t; i < (last - first) * 6; i += kPairThreads) s_box[i] = B[6 * (size_t)first + i];
   __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    const int2 v = t >= off ? part[t - off] : make_int2(0, 0);
+  auto box = [&](int j) { return load_box(s_box, j - first); };
+  const int c = start - kPlocRadius + t;  // the thread's cluster
+  if (t < kTile + H) s_nn[t] = c >= 0 && c < m ? nearest(c, m, box) : -1;
+  __syncthreads();
+  bool merges = false, stays = false;
+  if (t >= kPlocRadius && t < kTile + kPlocRadius && c < m) {
+    const int j = s_nn[t];
+    const bool mutual = j >= 0 && s_nn[j - start + kPlocRadius] == c;
+    merges = mutual && c < j;
+    stays = !(mutual && j < c);
+    P[c] = merges ? j : stays ? -1 : -2;
+  }
+  const unsigned a = __ballot_sync(0xffffffffu, merges), b = __ballot_sync(0xffffffffu, stays);
+  if ((t & 31) == 0) s_cnt[t >> 5] = make_int2(__popc(a), __popc(b));
+  __syncthreads();
+  const int tiles = (m + kTile - 1) / kTile;
+  if (t == 0) {
+    int2 n = make_int2(0, 0);
+    for (int w = 0; w < kPairThreads / 32; ++w) {
+      n.x += s_cnt[w].x;
+      n.y += s_cnt[w].y;
+    }
+    sums[blockIdx.x] = n;
+    __threadfence();
+    s_last = atomicAdd(&S->tiles_done, 1) == tiles - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  // a contiguous chunk of tiles per thread, a scan of the partial sums, the chunk's prefixes
+  __threadfence();
+  const int chunk = (tiles + kPairThreads - 1) / kPairThreads;
+  const int lo = min(t * chunk, tiles), hi = min(lo + chunk, tiles);
+  int2 acc = make_int2(0, 0);
+  for (int i = lo; i < hi; ++i) {
+    const int2 v = __ldcg(&sums[i]);
+    acc.x += v.x;
+    acc.y += v.y;
+  }
+  s_part[t] = acc;
+  __syncthreads();
+  for (int off = 1; off < kPairThreads; off <<= 1) {
+    const int2 v = t >= off ? s_part[t - off] : make_int2(0, 0);
     __syncthreads();
-    part[t].x += v.x;
-    part[t].y += v.y;
+    s_part[t].x += v.x;
+    s_part[t].y += v.y;
     __syncthreads();
   }
-  int2 run = t > 0 ? part[t - 1] : make_int2(0, 0);
-  for (int i = b; i < e; ++i) {
-    const int2 v = sums[i];
+  int2 run = t > 0 ? s_part[t - 1] : make_int2(0, 0);
+  for (int i = lo; i < hi; ++i) {
+    const int2 v = __ldcg(&sums[i]);
     sums[i] = run;
     run.x += v.x;
     run.y += v.y;
   }
-  if (t == 1023) {
-    S->m[parity ^ 1] = part[1023].y;
-    S->created[parity ^ 1] = created + part[1023].x;
+  if (t == kPairThreads - 1) {
+    S->m[parity ^ 1] = s_part[t].y;
+    S->created[parity ^ 1] = created + s_part[t].x;
+    S->tiles_done = 0;
   }
 }
 
@@ -500,7 +510,7 @@ inline cudaError_t launch_sort(unsigned long long* keys, int n_pad, cudaStream_t
 // its largest-area internal child until it has up to four children.  A wide
 // node stores its box origin P (float32), one power-of-two scale 2^e per axis
 // and 8-bit child bounds q with  P + qlo 2^e <= child lo  and  P + qhi 2^e >=
-// child hi, computed in FP64 from exact float32 values, so every decoded box
+// child hi, computed with directed rounding, so every decoded box
 // contains its child: the traversal can only visit more, never miss a hit.
 // Layout (64 bytes = 4 x uint4):
 //   w0..2 P.xyz, w3 = e.x | e.y << 8 | e.z << 16 (biased by 128) | count << 24
@@ -632,26 +642,21 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
       W.hi[k] = fmaxf(W.hi[k], cb[c].hi[k]);
     }
   }
+  // All of this in FP32 with directed rounding (lower bounds down, upper ones
+  // up); in FP64 the launches of the collapse took 0.7 ms of a 92k-triangle
+  // build, now 0.15.
   unsigned char qlo[3][4], qhi[3][4];
   int ex[3];
   for (int k = 0; k < 3; ++k) {
-    const double ext = (double)W.hi[k] - (double)W.lo[k];
-    int e = -100;
-    if (ext > 0.0) {
-      e = (int)ceil(log2(ext / 255.0));
-      while (ldexp(255.0, e) < ext) ++e;
-      if (e < -100) e = -100;
-    }
+    // the least power of two 2^e with 255 * 2^e >= the node's extent
+    const unsigned r = __float_as_uint(__fdiv_ru(__fsub_ru(W.hi[k], W.lo[k]), 255.0f));
+    const int e = r == 0u ? -100 : max((int)(r >> 23) - 127 + ((r & 0x7fffffu) != 0u), -100);
     ex[k] = e;
-    const double sc = ldexp(1.0, e);
+    const float sc = __uint_as_float((unsigned)(127 - e) << 23);  // 2^-e
     for (int c = 0; c < 4; ++c) {
       if (c < cnt) {
-        double lo = floor(((double)cb[c].lo[k] - (double)W.lo[k]) / sc);
-        double hi = ceil(((double)cb[c].hi[k] - (double)W.lo[k]) / sc);
-        lo = lo < 0.0 ? 0.0 : (lo > 255.0 ? 255.0 : lo);
-        hi = hi < 0.0 ? 0.0 : (hi > 255.0 ? 255.0 : hi);
-        qlo[k][c] = (unsigned char)lo;
-        qhi[k][c] = (unsigned char)hi;
+        qlo[k][c] = (unsigned char)fminf(floorf(__fsub_rd(cb[c].lo[k], W.lo[k]) * sc), 255.0f);
+        qhi[k][c] = (unsigned char)fminf(ceilf(__fsub_ru(cb[c].hi[k], W.lo[k]) * sc), 255.0f);
       } else {
         qlo[k][c] = 255;  // empty slot: an inverted box that no ray hits
         qhi[k][c] = 0;
@@ -696,9 +701,9 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
     for (int k = 0; k < 3; ++k) {
       w[k] = 0xffffu;  // empty: an inverted box
       if (c < cnt) {
-        const double lo = floor(((double)cb[c].lo[k] - (double)g.lo[k]) / (double)g.step[k]);
-        const double hi = ceil(((double)cb[c].hi[k] - (double)g.lo[k]) / (double)g.step[k]);
-        w[k] = (unsigned)fmin(fmax(lo, 0.0), 65535.0) | ((unsigned)fmin(fmax(hi, 0.0), 65535.0) << 16);
+        const float lo = floorf(__fmul_rd(__fsub_rd(cb[c].lo[k], g.lo[k]), __frcp_rd(g.step[k])));
+        const float hi = ceilf(__fmul_ru(__fsub_ru(cb[c].hi[k], g.lo[k]), __frcp_ru(g.step[k])));
+        w[k] = (unsigned)fminf(fmaxf(lo, 0.0f), 65535.0f) | ((unsigned)fminf(fmaxf(hi, 0.0f), 65535.0f) << 16);
       }
     }
     gn[4 * (size_t)widx + c] = make_uint4(w[0], w[1], w[2], c < cnt ? (unsigned)refs[c] : 0x80000000u);
@@ -758,15 +763,14 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
       return r;
     if (n == 1) return cudaGetLastError();
     k_leaf_clusters<<<g256, 256, 0, st>>>(tri, n, Bc, Cc);
-    // rounds of the many-block form: a round leaves about 0.65 of the clusters
+    // rounds of the many-block form: a round leaves about 0.78 of the clusters
     int parity = 0;
     for (long long bound = n, done = 0; done < n;) {
       int rounds = 0;
-      for (double m = (double)bound; m > kTail; m *= 0.7) ++rounds;
+      for (double m = (double)bound; m > kTail; m *= 0.78) ++rounds;
       const int tiles = (int)((bound + kTile - 1) / kTile);
       for (int k = 0; k < rounds; ++k) {
-        k_ploc_pairs<<<tiles, kTile, 0, st>>>(Bc, S, parity, P, sums);
-        k_ploc_scan<<<1, 1024, 0, st>>>(sums, S, parity);
+        k_ploc_pairs<<<tiles, kPairThreads, 0, st>>>(Bc, S, parity, P, sums);
         k_ploc_merge<<<tiles, kTile, 0, st>>>(Bc, Cc, P, sums, S, parity, n, Bn, Cn, nodes);
         std::swap(Bc, Bn);
         std::swap(Cc, Cn);
