@@ -490,7 +490,8 @@ __device__ __forceinline__ bool bin_step(const void* __restrict__ nodes, BinTrav
   return false;
 }
 
-// One visit of a 4-wide grid node (same contract as bin_step).  The boxes
+// One visit of a 4-wide grid node (same contract as bin_step, but the caller
+// counts the visits by the guard's fall).  The boxes
 // contain the FP32 ones, so a triangle that the FP32 tree tests is tested.
 // The nearest internal child is walked next (entry distances as ordered
 // integers with the child's index in the two low bits), the others are pushed
@@ -498,13 +499,12 @@ __device__ __forceinline__ bool bin_step(const void* __restrict__ nodes, BinTrav
 // costs 1% of the time.  An empty child has an inverted box, and leaf slot 0
 // as its reference in case a degenerate grid lets a ray in all the same.
 template <class LeafFn>
-__device__ __forceinline__ bool grid_step(const uint4* __restrict__ nodes, BinTrav& s, int* stack, int* visits,
-                                          int* err, LeafFn&& leaf) {
+__device__ __forceinline__ bool grid_step(const uint4* __restrict__ nodes, BinTrav& s, int* stack, int* err,
+                                          LeafFn&& leaf) {
   if (--s.guard < 0) {
     if (err) *err = 2;
     return true;
   }
-  ++*visits;
   const uint4* N = nodes + 4 * (size_t)(unsigned)s.node;
   uint4 c[4];
 #pragma unroll
@@ -531,8 +531,7 @@ __device__ __forceinline__ bool grid_step(const uint4* __restrict__ nodes, BinTr
       else if (err) *err = 1;
     }
   if (near != kNone) {
-    const unsigned a = near & 1u ? c[1].w : c[0].w, b = near & 1u ? c[3].w : c[2].w;
-    s.node = (int)(near & 2u ? b : a);
+    s.node = (int)(near & 2u ? (near & 1u ? c[3].w : c[2].w) : (near & 1u ? c[1].w : c[0].w));
     return false;
   }
   if (s.sp == 0) return true;

@@ -652,7 +652,7 @@ constexpr int kGridLeaves = GR_GRID_LEAVES;
 // of 4 warps per issue) beside 58% busy ALUs at 17 of 32 lanes.  The 4-wide
 // grid nodes halve the chain: 13.2 visits per ray instead of 26.0, and 20%
 // fewer instructions; k_trace on 129M rays of a 512^2 x 256 spp render of 91k
-// triangles went from 38.6 to 32.1 ms (binary nodes with FP16 boxes before;
+// triangles went from 38.6 to 31.7 ms (binary nodes with FP16 boxes before;
 // the same binary nodes on the grid: 37.8).  kGridLeaves 4 / 5 / 8: 34.4 /
 // 33.6 / 33.6 ms against 32.9 at 6; 2 / 3 / 4 visits between two looks at the
 // schedule: 35.4 / 34.0 / 32.9 ms against 32.5 at 6; 6 or 8 blocks per SM:
@@ -674,14 +674,13 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
   bool live = false;     // the lane holds a ray
   bool walking = false;  // ... whose node walk has not ended
   int np = 0, pl0 = 0, pl1 = 0, pl2 = 0;  // queued leaves (at most 3)
-  int exclude = -1;                        // the ray's s.exclude, kept for the queueing test
   // the lane's queued leaves: three registers, or kGridLeaves words of shared
   // memory for the 4-wide nodes, which can add four at a visit
   constexpr bool GRID = TREE == kTreeGrid;
   __shared__ int s_leaf[GRID ? kGridLeaves : 1][GRID ? GR_TRACE_BLOCK : 1];
   constexpr int kFull = GRID ? kGridLeaves - 3 : 2;  // a lane holding as many stops walking
   auto queue_leaf = [&](int leaf) {
-    if (leaf == exclude) return;
+    if (leaf == s.exclude) return;
     if (GRID) s_leaf[np][threadIdx.x] = leaf;
     else if (np == 0) pl0 = leaf;
     else if (np == 1) pl1 = leaf;
@@ -694,6 +693,9 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
     h.slot = s.slot;
     done(out, h);
     live = false;
+    // visits of the 4-wide walk: the guard's start was added with the ray (a
+    // counter of its own in the inner loop costs 3%)
+    if (GRID) visits -= s.guard;
   };
   // the warp's claimed group: its last `left` entries (from base + group - left) are unread
   const int group = n > GR_TRACE_BIG_QUEUE ? 64 : 32;
@@ -734,8 +736,8 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
         tri = S.tri;
         out = slot;
         np = 0;
-        exclude = x;
         live = walking = !bin_begin<TREE>(S, s, o, d, x, &refined, &tests);
+        if (GRID) visits += s.guard;
         if (!live) {
           live = true;
           finish();
@@ -764,7 +766,7 @@ __device__ __forceinline__ void lane_trace(const RenderParams& p, int n, int* cu
 #pragma unroll 1
     for (int k = 0; k < kSteps && live && walking && np < kFull; ++k) {
       if (GRID)
-        walking = !grid_step((const uint4*)nodes, s, stack, &visits, &err, queue_leaf);
+        walking = !grid_step((const uint4*)nodes, s, stack, &err, queue_leaf);
       else
         walking = !bin_step(nodes, s, stack, &visits, &err, queue_leaf);
       if (!walking && np == 0) finish();
