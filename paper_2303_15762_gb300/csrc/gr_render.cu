@@ -56,11 +56,11 @@ constexpr long long kMinDefaultPool = 1LL << 16;
 #ifndef GR_TRACE_BLOCK
 #define GR_TRACE_BLOCK 128
 #endif
-// shading: 4 blocks/SM (64 registers) for both Stokes counts.  The spills
-// this costs the 4-Stokes kernel are cheaper than the latency left exposed
-// with a quarter fewer resident warps (measured on both forms).
+// shading: 3 blocks/SM (80 registers) with 4 Stokes components, 4 with one:
+// on entries sorted by class, 18.0 against 19.4 ms at 4 blocks and 18.4 at 2
+// (4 Stokes), 5.0 against 5.2 ms at 3 (one)
 #ifndef GR_SHADE_MIN_BLOCKS
-#define GR_SHADE_MIN_BLOCKS 4
+#define GR_SHADE_MIN_BLOCKS 3
 #endif
 #ifndef GR_SHADE_MIN_BLOCKS_NS1
 #define GR_SHADE_MIN_BLOCKS_NS1 4
@@ -212,68 +212,10 @@ __device__ __forceinline__ void warp_count(unsigned long long* ctr, int v) {
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(ctr, (unsigned long long)v);
 }
 
-// Block-wide queue reservation with one atomic per block: returns this
-// thread's slot in the queue for `want` entries (exclusive scan over the
-// block's warps).  Every thread of the block must call it (uniform control
-// flow); the trailing barrier lets the shared words be reused by the next call.
-template <typename CT>
-__device__ __forceinline__ CT block_reserve(CT* counter, bool want) {
-  __shared__ int s_warp[8];
-  __shared__ CT s_base;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  const unsigned m = __ballot_sync(0xffffffffu, want);
-  if (lane == 0) s_warp[warp] = __popc(m);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int tot = 0;
-    for (int w = 0; w < nw; ++w) {
-      const int c = s_warp[w];
-      s_warp[w] = tot;
-      tot += c;
-    }
-    s_base = tot ? atomicAdd(counter, (CT)tot) : (CT)0;
-  }
-  __syncthreads();
-  const CT off = s_base + (CT)(s_warp[warp] + __popc(m & ((1u << lane) - 1u)));
-  __syncthreads();
-  return off;
-}
-
-// Two block-wide queue reservations with one set of barriers: this thread's
-// entries in queue a (for want_a) and in queue b (for want_b).  Uniform
-// control flow, as block_reserve.
-__device__ __forceinline__ int2 block_reserve2(int* counter_a, bool want_a, int* counter_b, bool want_b) {
-  __shared__ int s_wa[8], s_wb[8];
-  __shared__ int s_base[2];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  const unsigned ma = __ballot_sync(0xffffffffu, want_a), mb = __ballot_sync(0xffffffffu, want_b);
-  if (lane == 0) {
-    s_wa[warp] = __popc(ma);
-    s_wb[warp] = __popc(mb);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ta = 0, tb = 0;
-    for (int w = 0; w < nw; ++w) {
-      const int ca = s_wa[w], cb = s_wb[w];
-      s_wa[w] = ta;
-      s_wb[w] = tb;
-      ta += ca;
-      tb += cb;
-    }
-    s_base[0] = ta ? atomicAdd(counter_a, ta) : 0;
-    s_base[1] = tb ? atomicAdd(counter_b, tb) : 0;
-  }
-  __syncthreads();
-  const unsigned below = (1u << lane) - 1u;
-  const int2 off = make_int2(s_base[0] + s_wa[warp] + __popc(ma & below), s_base[1] + s_wb[warp] + __popc(mb & below));
-  __syncthreads();
-  return off;
-}
-
 // Block-wide reservation of n entries per thread (n >= 0) with one atomic per
 // block: returns the first of this thread's n entries (exclusive scan over the
-// block).  Uniform control flow, as block_reserve.
+// block).  Every thread of the block must call it (uniform control flow); the
+// trailing barrier lets the shared words be reused by the next call.
 template <typename CT>
 __device__ __forceinline__ CT block_reserve_n(CT* counter, int n) {
   __shared__ int s_warp[8];
@@ -1355,95 +1297,198 @@ __global__ void __launch_bounds__(256, MODE == 1   ? GR_SHADE_MIN_BLOCKS_HERO
   // queue counters for the next regen pass
   const int front = *(volatile int*)&p.ctr->tq_front;
   const int n = *(volatile int*)&p.ctr->tq_n;
-  for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
-    const int i = base + threadIdx.x;
-    bool want_shadow = false;
-    bool want_density = false;  // hero: the class lobe densities are deferred to k_density
-    int slot = -1;
-    if (i < n) {
-      slot = tq_entry(p, i, front);
-      int4 m = P.meta[slot];
-      const DevView& V = p.views[m.x];
-      const DevScene& S = p.scenes[V.scene_index];
-      float4 a0 = P.od0[slot], a1 = P.od1[slot];
-      const float2 hh = P.hit[slot];
-      float3 o = xyz(a0), d = xyz(a1);
-      float beta2 = a0.w, rho = a1.w;
-      const int kk = meta_k(m.z), seg = meta_seg(m.z), prev_delta = meta_delta(m.z);
-      const int WH = V.W * V.H;
-      const int cls = m.y / WH;  // the ticket's sample class (its bin without HERO)
-      const int pixel = m.y - cls * WH;
-      const int Qv = HERO ? V.Q : V.nb;
-      const int smp = class_first_sample(V, cls, Qv) + kk * Qv;
-      const int bin = HERO ? smp % V.nb : cls;
-      const int gh = HERO ? (bin - cls) / Qv : 0;  // the hero's member of the class
-      const float lambda = bin_lambda(V, bin);
-      const float cstep = HERO ? bin_step(V) : 0.0f;
-      const float kw = 2.0f * kPi / lambda;
-      const float s_ray2 = 1.0f / (2.0f * V.beta0 * V.beta0 * kw * kw);
-      float T[4][4];
-      float4 xfv = make_float4(0.0f, 0.0f, 0.0f, 1.0f), pt;
-      if (seg == 0) {
-        // camera segment (nothing stored by start_sample): identity Mueller
-        // matrix, no contribution yet, Stokes frame x axis = the camera's right
-        // vector made orthogonal to d, medium air
-        for (int r = 0; r < 4; ++r)
-          for (int c = 0; c < 4; ++c) T[r][c] = r == c ? 1.0f : 0.0f;
-        const float3 xf0 = NS == 1 && !ANISO ? f3(0.0f, 0.0f, 0.0f) : normalize(V.right - dot(V.right, d) * d);
-        xfv = make_float4(xf0.x, xf0.y, xf0.z, 1.0f);
-        pt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      } else {
-        if (NS == 1) {
-          const float4 t0 = P.tp[0][slot];
-          T[0][0] = t0.x;
-          xfv.w = t0.y;  // the medium's index rides in the unused word of the scalar throughput
+  // Entries are shaded in the order of what their segment met: a block takes a
+  // chunk of the queue, classes its entries (grating, rough lobe, other
+  // surface, escape) by their hits, and shades them class by class, so that
+  // the lanes of a warp mostly take the same branches.  Without the sort half
+  // of a warp's lanes (the escapes) waited for the others: 24 of 32 lanes
+  // active instead of 14 and 38% fewer instructions, which leaves the kernel
+  // bound by the latency of its loads (26% issue): 18.8 -> 18.0 ms on the 512^2
+  // x 256 spp render, hero 6.95 -> 6.2 ms (256^2 x 128 spp), a batch of 8 views
+  // 5.5 -> 5.0 ms.  Slot state is read past L1 (__ldcg), which keeps it for
+  // tables, triangles and spills; evict-first loads lose the half sectors that
+  // another warp reads (20.3 ms).
+  // Next-event and density requests are listed in shared memory and appended
+  // to their queues once per chunk, one atomic each.
+  constexpr int kPer = HERO ? 2 : 4, kChunk = kPer * 256, kClasses = 4;
+  __shared__ int s_list[kChunk];
+  __shared__ unsigned short s_sq[kChunk], s_dq[HERO ? kChunk : 1];
+  __shared__ short s_cnt[kClasses * kPer * 8];
+  __shared__ int s_n[4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  // short queues are spread over all blocks first
+  const int per = max(1, min(kPer, (n + (int)(gridDim.x * blockDim.x) - 1) / (int)(gridDim.x * blockDim.x)));
+  const int chunk = per * blockDim.x;
+  for (int base = blockIdx.x * chunk; base < n; base += gridDim.x * chunk) {
+    int cslot[kPer], ckey[kPer];  // slot; class << 8 | rank among the warp's entries of that class
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      if (j >= per) break;
+      const int i = base + j * blockDim.x + threadIdx.x;
+      int cl = kClasses;
+      cslot[j] = -1;
+      if (i < n) {
+        const int sl = tq_entry(p, i, front);
+        cslot[j] = sl;
+        const int hs = __float_as_int(P.hit[sl].y);
+        cl = 3;
+        if (hs >= 0) {
+          const DevScene& S = p.scenes[p.views[P.meta[sl].x].scene_index];
+          const int ty = S.mats[S.tri_mat[hs]].type;
+          cl = ty == GR_MAT_GRATING ? 0 : ty == GR_MAT_ROUGH ? 1 : 2;
+        }
+      }
+      int rank = 0;
+#pragma unroll
+      for (int c = 0; c < kClasses; ++c) {
+        const unsigned m = __ballot_sync(0xffffffffu, cl == c);
+        if (cl == c) rank = __popc(m & below);
+        if (lane == c) s_cnt[(c * per + j) * warps + warp] = (short)__popc(m);
+      }
+      ckey[j] = cl << 8 | rank;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      // exclusive prefix over (class, j, warp)
+      const int tot = kClasses * per * warps, each = (tot + 31) / 32;
+      int sum = 0;
+      for (int k = 0; k < each; ++k) {
+        const int e = lane * each + k;
+        if (e < tot) sum += s_cnt[e];
+      }
+      int incl = sum;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+      }
+      int run = incl - sum;
+      for (int k = 0; k < each; ++k) {
+        const int e = lane * each + k;
+        if (e < tot) {
+          const int v = s_cnt[e];
+          s_cnt[e] = (short)run;
+          run += v;
+        }
+      }
+      if (lane < 4) s_n[lane] = 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      if (j >= per) break;
+      const int cl = ckey[j] >> 8;
+      if (cl < kClasses) s_list[s_cnt[(cl * per + j) * warps + warp] + (ckey[j] & 255)] = cslot[j];
+    }
+    __syncthreads();
+    const int cnt = min(chunk, n - base);
+    for (int q0 = 0; q0 < cnt; q0 += blockDim.x) {
+      const int q = q0 + threadIdx.x;
+      bool want_shadow = false;
+      bool want_density = false;  // hero: the class lobe densities are deferred to k_density
+      if (q < cnt) {
+        const int slot = s_list[q];
+        int4 m = __ldcg(&P.meta[slot]);
+        const DevView& V = p.views[m.x];
+        const DevScene& S = p.scenes[V.scene_index];
+        float4 a0 = __ldcg(&P.od0[slot]), a1 = __ldcg(&P.od1[slot]);
+        const float2 hh = __ldcg(&P.hit[slot]);
+        float3 o = xyz(a0), d = xyz(a1);
+        float beta2 = a0.w, rho = a1.w;
+        const int kk = meta_k(m.z), seg = meta_seg(m.z), prev_delta = meta_delta(m.z);
+        const int WH = V.W * V.H;
+        const int cls = m.y / WH;  // the ticket's sample class (its bin without HERO)
+        const int pixel = m.y - cls * WH;
+        const int Qv = HERO ? V.Q : V.nb;
+        const int smp = class_first_sample(V, cls, Qv) + kk * Qv;
+        const int bin = HERO ? smp % V.nb : cls;
+        const int gh = HERO ? (bin - cls) / Qv : 0;  // the hero's member of the class
+        const float lambda = bin_lambda(V, bin);
+        const float cstep = HERO ? bin_step(V) : 0.0f;
+        const float kw = 2.0f * kPi / lambda;
+        const float s_ray2 = 1.0f / (2.0f * V.beta0 * V.beta0 * kw * kw);
+        float T[4][4];
+        float4 xfv = make_float4(0.0f, 0.0f, 0.0f, 1.0f), pt;
+        if (seg == 0) {
+          // camera segment (nothing stored by start_sample): identity Mueller
+          // matrix, no contribution yet, Stokes frame x axis = the camera's right
+          // vector made orthogonal to d, medium air
+          for (int r = 0; r < 4; ++r)
+            for (int c = 0; c < 4; ++c) T[r][c] = r == c ? 1.0f : 0.0f;
+          const float3 xf0 = NS == 1 && !ANISO ? f3(0.0f, 0.0f, 0.0f) : normalize(V.right - dot(V.right, d) * d);
+          xfv = make_float4(xf0.x, xf0.y, xf0.z, 1.0f);
+          pt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         } else {
-          for (int r = 0; r < 4; ++r) {
-            float4 v = P.tp[r][slot];
-            T[r][0] = v.x;
-            T[r][1] = v.y;
-            T[r][2] = v.z;
-            T[r][3] = v.w;
+          if (NS == 1) {
+            const float4 t0 = __ldcg(&P.tp[0][slot]);
+            T[0][0] = t0.x;
+            xfv.w = t0.y;  // the medium's index rides in the unused word of the scalar throughput
+          } else {
+            for (int r = 0; r < 4; ++r) {
+              float4 v = __ldcg(&P.tp[r][slot]);
+              T[r][0] = v.x;
+              T[r][1] = v.y;
+              T[r][2] = v.z;
+              T[r][3] = v.w;
+            }
           }
+          if (NS == 4) xfv = __ldcg(&P.xf[slot]);
+          if (NS == 1 && ANISO) {  // the footprint's frame
+            const float4 f = P.xf[slot];
+            xfv = make_float4(f.x, f.y, f.z, xfv.w);
+          }
+          pt = __ldcg(&P.part[slot]);
         }
-        if (NS == 4) xfv = P.xf[slot];
-        if (NS == 1 && ANISO) {  // the footprint's frame
-          const float4 f = P.xf[slot];
-          xfv = make_float4(f.x, f.y, f.z, xfv.w);
+        // anisotropic footprint: isotropic beta0^2 I on the camera segment
+        AK K{beta2, 0.0f, beta2, 0.0f, 0.0f, 0.0f};
+        if (ANISO && seg > 0) {
+          const float4 k0 = P.ak0[slot], k1 = P.ak1[slot];
+          K = AK{k0.x, k0.y, k0.z, k0.w, k1.x, k1.y};
         }
-        pt = P.part[slot];
-      }
-      // anisotropic footprint: isotropic beta0^2 I on the camera segment
-      AK K{beta2, 0.0f, beta2, 0.0f, 0.0f, 0.0f};
-      if (ANISO && seg > 0) {
-        const float4 k0 = P.ak0[slot], k1 = P.ak1[slot];
-        K = AK{k0.x, k0.y, k0.z, k0.w, k1.x, k1.y};
-      }
-      float hq[4] = {1.0f, 1.0f, 1.0f, 1.0f};
-      if (HERO && seg > 0) {
-        const float4 q4 = P.hq[slot];
-        hq[0] = q4.x;
-        hq[1] = q4.y;
-        hq[2] = q4.z;
-        hq[3] = q4.w;
-      }
-      constexpr bool WAVE = true;
+        float hq[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+        if (HERO && seg > 0) {
+          const float4 q4 = P.hq[slot];
+          hq[0] = q4.x;
+          hq[1] = q4.y;
+          hq[2] = q4.z;
+          hq[3] = q4.w;
+        }
+        constexpr bool WAVE = true;
 #include "gr_shade_segment.cuh"
-      P.part[slot] = pt;
-      if (done) {
-        P.meta[slot] = make_int4(m.x, m.y, meta_pack(kk, seg, ST_DONE, 0), m.w);
-        P.st8[slot] = ST_DONE;
+        P.part[slot] = pt;
+        if (done) {
+          P.meta[slot] = make_int4(m.x, m.y, meta_pack(kk, seg, ST_DONE, 0), m.w);
+          P.st8[slot] = ST_DONE;
+        }
+      }
+      const unsigned mw = __ballot_sync(0xffffffffu, want_shadow);
+      if (mw) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&s_n[0], __popc(mw));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (want_shadow) s_sq[at + __popc(mw & below)] = (unsigned short)q;
+      }
+      if (HERO) {
+        const unsigned md = __ballot_sync(0xffffffffu, want_density);
+        if (md) {
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&s_n[1], __popc(md));
+          at = __shfl_sync(0xffffffffu, at, 0);
+          if (want_density) s_dq[at + __popc(md & below)] = (unsigned short)q;
+        }
       }
     }
-    if (HERO) {
-      // the next-event and density queues with one set of barriers
-      const int2 q = block_reserve2(&p.ctr->sq_count, want_shadow, &p.ctr->dq_count, want_density);
-      if (want_shadow) P.sq[q.x] = slot;
-      if (want_density) P.dq[q.y] = slot;
-    } else {
-      const int q = block_reserve<int>(&p.ctr->sq_count, want_shadow);
-      if (want_shadow) P.sq[q] = slot;
+    __syncthreads();
+    const int nsq = s_n[0], ndq = HERO ? s_n[1] : 0;
+    if (nsq > 0 || ndq > 0) {
+      if (threadIdx.x == 0) s_n[2] = nsq ? atomicAdd(&p.ctr->sq_count, nsq) : 0;
+      if (HERO && threadIdx.x == 32 % blockDim.x) s_n[3] = ndq ? atomicAdd(&p.ctr->dq_count, ndq) : 0;
+      __syncthreads();
+      for (int k = threadIdx.x; k < nsq; k += blockDim.x) P.sq[s_n[2] + k] = s_list[s_sq[k]];
+      for (int k = threadIdx.x; k < ndq; k += blockDim.x) P.dq[s_n[3] + k] = s_list[s_dq[k]];
     }
+    __syncthreads();
   }
 }
 
