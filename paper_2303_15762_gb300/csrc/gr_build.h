@@ -86,6 +86,7 @@ struct RenderParams {
   const TableRow* rows;
   const void* table_vals;
   const float* table_vals32;  // the same values in FP32 (== table_vals for FP32 tables)
+  const double* table_vals64; // and in FP64 (null in gr_render_static)
   int table_dtype;
   int table_smem;        // 1 if the order table is staged in shared memory
   int table_rows;

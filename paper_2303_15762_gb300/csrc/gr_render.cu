@@ -1173,17 +1173,25 @@ struct TableRound<__nv_bfloat16> {
 // Grating order j (Eq. K_grating): cumulative J_j(pi h / lambda)^2 over the
 // propagating orders (|t_mir + j lambda/Lambda g|^2 < 1), renormalised unless
 // `renorm` is false; returns the first j whose cumulative sum exceeds
-// u * total, or 0x7fffffff if none does.
+// u * total, or 0x7fffffff if none does.  The squares come from the FP64 table
+// vals64 (k_tables) or, without one (gr_render_static's descriptors must not
+// grow), from the series.  One such decision holds up a warp, and with it the
+// block, for the whole of its serial FP64 work: the ~2 x 20 series cost
+// ~100 us, which set the length of small renders (64^2 x 64 spp grating 161 ->
+// 47 us with the table) and kept the blocks of k_shade at their barriers (18.0
+// -> 16.4 ms on the 512^2 x 256 spp render, with 22k such decisions).
 __device__ __noinline__ int grating_pick_fp64(double lam_d, float height_um, int jm, float3 t_mir, float step,
-                                              float3 gt, bool renorm, float u) {
+                                              float3 gt, bool renorm, float u, const double* __restrict__ vals64) {
   const double xarg = kPiD * (double)height_um / lam_d;
+  auto weight = [&](int j) {
+    if (vals64) return __ldg(vals64 + (j < 0 ? -j : j));
+    const double J = bessel_j_d(j, xarg);
+    return J * J;
+  };
   double tot_d = 0.0;
   for (int j = -jm; j <= jm; ++j) {
     const float3 tj = t_mir + ((float)j * step) * gt;
-    if (dot(tj, tj) < 1.0f) {
-      const double J = bessel_j_d(j, xarg);
-      tot_d += J * J;
-    }
+    if (dot(tj, tj) < 1.0f) tot_d += weight(j);
   }
   if (!renorm) tot_d = 1.0;
   const double tgt = (double)u * tot_d;
@@ -1191,13 +1199,21 @@ __device__ __noinline__ int grating_pick_fp64(double lam_d, float height_um, int
   for (int j = -jm; j <= jm; ++j) {
     const float3 tj = t_mir + ((float)j * step) * gt;
     if (dot(tj, tj) < 1.0f) {
-      const double J = bessel_j_d(j, xarg);
-      cd += J * J;
+      cd += weight(j);
       if (cd > tgt) return j;
     }
   }
   return 0x7fffffff;
 }
+
+// 1 / m for m < 128 (the term counts of g <= kGCont).
+struct RcpTable {
+  double r[128];
+  constexpr RcpTable() : r() {
+    for (int m = 1; m < 128; ++m) r[m] = 1.0 / m;
+  }
+};
+__constant__ RcpTable c_rcp = RcpTable();
 
 // Rough-surface term count m ~ Poisson(g), g = (2 k sigma_h cos_i)^2: the
 // first m whose cumulative Poisson probability exceeds u (at most 1000).
@@ -1209,7 +1225,7 @@ __device__ __noinline__ int poisson_pick_fp64(double lam_d, float sigma_h_um, fl
   int mi = 0;
   while ((double)u >= cd && mi < 1000) {
     ++mi;
-    pd *= gd / mi;
+    pd *= mi < 128 ? gd * c_rcp.r[mi] : gd / mi;  // no FP64 division in the serial chain
     cd += pd;
   }
   return mi;
@@ -1877,9 +1893,11 @@ __device__ __forceinline__ __half table_store<__half>(float v) { return __float2
 template <>
 __device__ __forceinline__ __nv_bfloat16 table_store<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
-// vals32 (FP32 copy for re-decisions) is null when TT is float.
+// vals32 (FP32 copy for re-decisions) is null when TT is float; vals64 (FP64
+// copy for the last re-decision) may be null.
 template <typename TT>
-__global__ void k_tables(const TableBuildRow* rows, int n_rows, const DevView* views, TT* vals, float* vals32) {
+__global__ void k_tables(const TableBuildRow* rows, int n_rows, const DevView* views, TT* vals, float* vals32,
+                         double* vals64) {
   int r = blockIdx.x;
   if (r >= n_rows) return;
   const TableBuildRow R = rows[r];
@@ -1887,9 +1905,11 @@ __global__ void k_tables(const TableBuildRow* rows, int n_rows, const DevView* v
   const double lam = bin_lambda_d(V, R.bin);
   const double x = kPiD * (double)R.height_um / lam;  // h k / 2
   for (int j = threadIdx.x; j <= R.jmax; j += blockDim.x) {
-    const float v = order_weight(j, x);
+    const double J = bessel_j_d(j, x), w = J * J;
+    const float v = (float)w;  // as order_weight
     vals[R.offset + j] = table_store<TT>(v);
     if (vals32) vals32[R.offset + j] = v;
+    if (vals64) vals64[R.offset + j] = w;
   }
 }
 
@@ -2291,6 +2311,7 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
   const size_t o_brows = take(sizeof(TableBuildRow) * std::max<size_t>(plan.build_rows.size(), 1));
   const size_t o_vals = take(tsize * std::max(plan.vals_count, 1));
   const size_t o_vals32 = o.table_dtype == GR_TABLE_F32 ? o_vals : take(sizeof(float) * std::max(plan.vals_count, 1));
+  const size_t o_vals64 = take(sizeof(double) * std::max(plan.vals_count, 1));
   const size_t o_f4 = take(sizeof(float4) * (size_t)P * 14);
   const size_t o_hit = take(sizeof(float2) * (size_t)P * 2);  // hit, shh
   const size_t o_meta = take(sizeof(int4) * (size_t)P);
@@ -2332,6 +2353,7 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
   p.rows = (const TableRow*)(base + o_rows);
   p.table_vals = base + o_vals;
   p.table_vals32 = (const float*)(base + o_vals32);
+  p.table_vals64 = (const double*)(base + o_vals64);
   p.table_dtype = o.table_dtype;
   p.table_rows = (int)plan.rows.size();
   p.table_vals_count = plan.vals_count;
@@ -2401,12 +2423,14 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
                           cudaMemcpyHostToDevice, st));
     const TableBuildRow* br = (const TableBuildRow*)(base + o_brows);
     const int nr = (int)plan.build_rows.size();
+    double* vals64 = (double*)(base + o_vals64);
     if (o.table_dtype == GR_TABLE_F32)
-      k_tables<float><<<nr, 64, 0, st>>>(br, nr, p.views, (float*)(base + o_vals), nullptr);
+      k_tables<float><<<nr, 64, 0, st>>>(br, nr, p.views, (float*)(base + o_vals), nullptr, vals64);
     else if (o.table_dtype == GR_TABLE_F16)
-      k_tables<__half><<<nr, 64, 0, st>>>(br, nr, p.views, (__half*)(base + o_vals), (float*)(base + o_vals32));
+      k_tables<__half><<<nr, 64, 0, st>>>(br, nr, p.views, (__half*)(base + o_vals), (float*)(base + o_vals32), vals64);
     else
-      k_tables<__nv_bfloat16><<<nr, 64, 0, st>>>(br, nr, p.views, (__nv_bfloat16*)(base + o_vals), (float*)(base + o_vals32));
+      k_tables<__nv_bfloat16><<<nr, 64, 0, st>>>(br, nr, p.views, (__nv_bfloat16*)(base + o_vals), (float*)(base + o_vals32),
+                                               vals64);
     f->launches += 1;
   }
   if (!paths) GR_CK(cudaMemsetAsync(p.pool.meta, 0, sizeof(int4) * (size_t)P, st));
@@ -2865,11 +2889,11 @@ gr_status render_static_impl(gr_scene* const* scenes, int n_scenes, const gr_vie
     const TableBuildRow* br = (const TableBuildRow*)(base + o_brows);
     const int nr = (int)brows.size();
     if (o.table_dtype == GR_TABLE_F32)
-      k_tables<float><<<nr, 64, 0, st>>>(br, nr, p.views, (float*)(base + o_vals), nullptr);
+      k_tables<float><<<nr, 64, 0, st>>>(br, nr, p.views, (float*)(base + o_vals), nullptr, nullptr);
     else if (o.table_dtype == GR_TABLE_F16)
-      k_tables<__half><<<nr, 64, 0, st>>>(br, nr, p.views, (__half*)(base + o_vals), (float*)(base + o_vals32));
+      k_tables<__half><<<nr, 64, 0, st>>>(br, nr, p.views, (__half*)(base + o_vals), (float*)(base + o_vals32), nullptr);
     else
-      k_tables<__nv_bfloat16><<<nr, 64, 0, st>>>(br, nr, p.views, (__nv_bfloat16*)(base + o_vals), (float*)(base + o_vals32));
+      k_tables<__nv_bfloat16><<<nr, 64, 0, st>>>(br, nr, p.views, (__nv_bfloat16*)(base + o_vals), (float*)(base + o_vals32), nullptr);
   }
   GR_SK(cudaGetLastError());
   // --- launch shapes (same rule as gr_render)

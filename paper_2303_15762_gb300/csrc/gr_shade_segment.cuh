@@ -240,7 +240,8 @@
                                     [&](int a) { return __ldg(p.table_vals32 + row.offset + a); }, ambiguous);
           if (ambiguous) {
             atomicAdd(&p.ctr->ref_lobe, 1ull);
-            pick = grating_pick_fp64(bin_lambda_d(V, bin), M.height_um, jm, t_mir, step, gt, renorm, u.x);
+            pick = grating_pick_fp64(bin_lambda_d(V, bin), M.height_um, jm, t_mir, step, gt, renorm, u.x,
+                                     p.table_vals64 ? p.table_vals64 + row.offset : nullptr);
           }
           if (pick == 0x7fffffff) {
             alive = false;
