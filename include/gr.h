@@ -236,6 +236,9 @@ typedef struct {
  * Errors: GR_E_INVALID (null/negative sizes, material index out of range,
  * unknown material or light type), GR_E_OOM, GR_E_CUDA. */
 gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene** out);
+/* Free the scene.  Synchronises its device (a render may still read it).  The
+ * library keeps up to 256 MB of freed device memory for its next calls (512 MB
+ * while scenes or frames live) and gives it back when an allocation fails. */
 gr_status gr_scene_destroy(gr_scene* scene);
 /* Device bytes the scene holds (triangles, BVH layouts, materials, lights,
  * emitters); host-side bookkeeping, no CUDA call.  Errors: GR_E_INVALID. */

@@ -155,28 +155,14 @@ def pack_views(views):
     return arr
 
 
-def _pack_materials(rows):
-    rows = np.asarray(rows, dtype=np.float32).reshape(-1, 16)
-    arr = (gr_material * max(1, len(rows)))()
-    for i, r in enumerate(rows):
-        m = arr[i]
-        m.type, m.fresnel = int(r[0]), int(r[1])
-        m.n_re, m.n_im, m.period_um, m.height_um = float(r[2]), float(r[3]), float(r[4]), float(r[5])
-        m.gdir[:] = [float(x) for x in r[6:9]]
-        m.sigma_h_um, m.corr_len_um, m.Le, m.coh_len_um = float(r[9]), float(r[10]), float(r[11]), float(r[12])
-        m.cauchy_b_um2 = float(r[13])
-    return arr, len(rows)
-
-
-def _pack_lights(rows):
-    rows = np.asarray(rows, dtype=np.float32).reshape(-1, 8)
-    arr = (gr_light * max(1, len(rows)))()
-    for i, r in enumerate(rows):
-        L = arr[i]
-        L.type = int(r[0])
-        L.dir[:] = [float(x) for x in r[1:4]]
-        L.E, L.coh_len_um = float(r[4]), float(r[5])
-    return arr, len(rows)
+def _pack_rows(rows, words, ints):
+    """Rows of the generators as the C structs: the same words in the same
+    order, the first `ints` as integers, the reserved last two zero."""
+    rows = np.asarray(rows, dtype=np.float32).reshape(-1, words)
+    out = np.zeros((max(1, len(rows)), words), dtype=np.float32)
+    out[:len(rows), :words - 2] = rows[:, :words - 2]
+    out.view(np.int32)[:len(rows), :ints] = rows[:, :ints].astype(np.int32)
+    return out, len(rows)
 
 
 class Scene:
@@ -187,10 +173,9 @@ class Scene:
         self._h = ctypes.c_void_p()
         verts = np.ascontiguousarray(scene["verts"], dtype=np.float32).reshape(-1, 9)
         tri_mat = np.ascontiguousarray(scene["tri_mat"], dtype=np.int32)
-        mats, n_mats = _pack_materials(scene["mats"])
-        lights, n_lights = _pack_lights(scene["lights"])
-        desc = gr_scene_desc(len(tri_mat), _ptr(verts), _ptr(tri_mat), n_mats,
-                             ctypes.cast(mats, ctypes.c_void_p), n_lights, ctypes.cast(lights, ctypes.c_void_p))
+        mats, n_mats = _pack_rows(scene["mats"], 16, 2)    # gr_material
+        lights, n_lights = _pack_rows(scene["lights"], 8, 1)  # gr_light
+        desc = gr_scene_desc(len(tri_mat), _ptr(verts), _ptr(tri_mat), n_mats, _ptr(mats), n_lights, _ptr(lights))
         self.n_tris = len(tri_mat)
         self.host_bytes = verts.nbytes + tri_mat.nbytes + n_mats * 64 + n_lights * 32
         _check(L.gr_scene_create(ctypes.byref(desc), stream or current_stream(), ctypes.byref(self._h)))

@@ -386,7 +386,7 @@ cudaError_t run_aperture(int dim, const void* kernel, int n_det, const double* x
   const size_t o_out = o_part + (sizeof(double) * (size_t)n_det * n_split + 255) / 256 * 256;
   unsigned char* d = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&d, o_out + sizeof(double) * (size_t)n_det, st);
+  cudaError_t e = dev_alloc((void**)&d, o_out + sizeof(double) * (size_t)n_det, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d, x0_host, b_x0, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d + o_ap, h.data(), smem, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && ms) e = cudaEventCreate(&e0);

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -21,6 +22,119 @@ cudaError_t debug_rng_impl(uint32_t seed, uint32_t view, uint32_t pixel, uint32_
                            uint32_t* host_out, cudaStream_t st);
 gr_status render_static_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc* vd, int n_views,
                              const gr_render_opts& o, float* accum, cudaStream_t st, std::string& err);
+}  // namespace gr
+
+namespace gr {
+
+// One memory pool per device, created at its first use.  A pool that gives its
+// memory back at every synchronisation (the default one) makes each call map
+// and unmap it again: ~90 us per allocation of a few KB, 1 ms for 500 MB.  This
+// one keeps up to kPoolKeep bytes while scenes or frames live, and at most
+// kPoolIdle once the last of them is gone; what it keeps is given back when an
+// allocation of the library fails.  Allocation and release are stream-ordered
+// and safe from several threads.
+namespace {
+constexpr size_t kPoolKeep = 512u << 20, kPoolIdle = 256u << 20;
+struct LibPool {
+  std::mutex m;
+  cudaMemPool_t pool = nullptr;
+  bool tried = false;
+  long long live = 0;  // scenes and frames of the device
+};
+LibPool g_pools[64];
+
+cudaMemPool_t pool_of(int dev) {
+  if (dev < 0 || dev >= 64) return nullptr;
+  LibPool& L = g_pools[dev];
+  std::lock_guard<std::mutex> lock(L.m);
+  if (!L.tried) {
+    L.tried = true;
+    cudaMemPoolProps pr = {};
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    pr.location.id = dev;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&L.pool, &pr) != cudaSuccess ||
+        cudaMemPoolSetAttribute(L.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      L.pool = nullptr;
+    }
+  }
+  return L.pool;
+}
+
+// A scene or frame of device dev comes (+1) or goes (-1).
+void count_object(int dev, int change) {
+  const cudaMemPool_t pool = pool_of(dev);
+  if (!pool) return;
+  LibPool& L = g_pools[dev];
+  std::lock_guard<std::mutex> lock(L.m);
+  L.live += change;
+  if (L.live == 0 && cudaMemPoolTrimTo(pool, kPoolIdle) != cudaSuccess) cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  const cudaMemPool_t pool = pool_of(dev);
+  if (!pool) return cudaMallocAsync(p, bytes, st);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  if (e == cudaSuccess) return e;
+  cudaGetLastError();
+  if (e == cudaErrorMemoryAllocation) {
+    // what the pool keeps may be in the way, in pieces too small
+    cudaStreamSynchronize(st);
+    cudaMemPoolTrimTo(pool, 0);
+    cudaGetLastError();
+    return cudaMallocFromPoolAsync(p, bytes, pool, st);
+  }
+  return cudaMallocAsync(p, bytes, st);  // the pool is gone (its device was reset)
+}
+
+// Pinned counters of a frame (two Counters): pairs of one 64-pair block, kept
+// for the process (19 KB), since pinning host memory takes ~120 us each way;
+// frames beyond 64 pin their own.
+namespace {
+std::mutex g_pin_m;
+Counters* g_pin = nullptr;
+unsigned long long g_pin_used = 0;
+}  // namespace
+
+cudaError_t pin_counters(Counters** out) {
+  std::lock_guard<std::mutex> lock(g_pin_m);
+  if (g_pin) {
+    // a device reset unpins it: then another block is pinned
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, g_pin) != cudaSuccess || a.type != cudaMemoryTypeHost) {
+      cudaGetLastError();
+      g_pin = nullptr;
+      g_pin_used = 0;
+    }
+  }
+  if (!g_pin) {
+    const cudaError_t e = cudaHostAlloc((void**)&g_pin, sizeof(Counters) * 2 * 64, cudaHostAllocPortable);
+    if (e != cudaSuccess) {
+      g_pin = nullptr;
+      return e;
+    }
+  }
+  for (int i = 0; i < 64; ++i)
+    if (!((g_pin_used >> i) & 1ull)) {
+      g_pin_used |= 1ull << i;
+      *out = g_pin + 2 * i;
+      return cudaSuccess;
+    }
+  return cudaHostAlloc((void**)out, sizeof(Counters) * 2, cudaHostAllocPortable);
+}
+
+void unpin_counters(Counters* c) {
+  std::lock_guard<std::mutex> lock(g_pin_m);
+  if (g_pin && c >= g_pin && c < g_pin + 2 * 64)
+    g_pin_used &= ~(1ull << ((c - g_pin) / 2));
+  else
+    cudaFreeHost(c);
+}
 }  // namespace gr
 
 namespace {
@@ -110,12 +224,12 @@ gr_status frame_make(const char* who, const gr_view_desc* views, int32_t n_views
   if (acc) {
     F->acc = acc;
   } else {
-    e = cudaMallocAsync(&F->acc, sizeof(float) * total * 2, st);
+    e = gr::dev_alloc(&F->acc, sizeof(float) * total * 2, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(F->acc, 0, sizeof(float) * total * 2, st);
   }
-  if (e == cudaSuccess) e = cudaMallocAsync(&F->ctr, sizeof(gr::Counters), st);
+  if (e == cudaSuccess) e = gr::dev_alloc(&F->ctr, sizeof(gr::Counters), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(F->ctr, 0, sizeof(gr::Counters), st);
-  if (e == cudaSuccess) e = cudaHostAlloc(&F->ctr_host, sizeof(gr::Counters) * 2, cudaHostAllocDefault);
+  if (e == cudaSuccess) e = gr::pin_counters(&F->ctr_host);
   if (e != cudaSuccess) {
     if (F->acc && F->owns_acc) cudaFreeAsync(F->acc, st);
     if (F->ctr) cudaFreeAsync(F->ctr, st);
@@ -123,6 +237,7 @@ gr_status frame_make(const char* who, const gr_view_desc* views, int32_t n_views
     return cuda_fail(e, w.c_str());
   }
   std::memset(F->ctr_host, 0, sizeof(gr::Counters) * 2);
+  gr::count_object(dev, 1);
   *out = F;
   return GR_OK;
 }
@@ -262,7 +377,7 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
   bool grid_ok = false;
   const size_t o_grid = take(sizeof(uint4) * 4 * (size_t)std::max(n - 1, 0));
   int n_wide = 0;
-  cudaError_t e = cudaMallocAsync(&S->mem, off, st);
+  cudaError_t e = gr::dev_alloc(&S->mem, off, st);
   if (e != cudaSuccess) {
     delete S;
     return cuda_fail(e, "gr_scene_create: device allocation");
@@ -273,8 +388,8 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
   gr_status status = GR_OK;
   do {
     if (n > 0) {
-      if ((e = cudaMallocAsync(&verts_d, sizeof(float) * 9 * (size_t)n, st)) != cudaSuccess) break;
-      if ((e = cudaMallocAsync(&tmat_in, sizeof(int) * (size_t)n, st)) != cudaSuccess) break;
+      if ((e = gr::dev_alloc(&verts_d, sizeof(float) * 9 * (size_t)n, st)) != cudaSuccess) break;
+      if ((e = gr::dev_alloc(&tmat_in, sizeof(int) * (size_t)n, st)) != cudaSuccess) break;
       if ((e = cudaMemcpyAsync(verts_d, desc->verts, sizeof(float) * 9 * (size_t)n, cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
       if ((e = cudaMemcpyAsync(tmat_in, desc->tri_mat, sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
     }
@@ -323,6 +438,7 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
   D.emitter_tris = (const float4*)(b + o_etri);
   S->keys = (unsigned long long*)(b + o_keys);
   S->bytes = off;
+  gr::count_object(S->device, 1);
   *out = S;
   return GR_OK;
 }
@@ -335,7 +451,15 @@ gr_status gr_scene_bytes(const gr_scene* scene, size_t* bytes_out) {
 
 gr_status gr_scene_destroy(gr_scene* scene) {
   if (!scene) return fail(GR_E_INVALID, "gr_scene_destroy: null scene");
+  // a render may still read the scene (gr_render returns before its work is
+  // done): its memory goes back to the pool only after that
+  int dev = -1;
+  const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != scene->device;
+  if (other) cudaSetDevice(scene->device);
+  cudaDeviceSynchronize();
   if (scene->mem) cudaFree(scene->mem);
+  gr::count_object(scene->device, -1);
+  if (other) cudaSetDevice(dev);
   delete scene;
   return GR_OK;
 }
@@ -393,9 +517,10 @@ gr_status gr_frame_release(gr_frame* f) {
   if (f->acc && f->owns_acc) cudaFree(f->acc);
   if (f->scratch) cudaFree(f->scratch);
   if (f->ctr) cudaFree(f->ctr);
-  if (f->ctr_host) cudaFreeHost(f->ctr_host);
+  if (f->ctr_host) gr::unpin_counters(f->ctr_host);
   if (f->graph_exec) cudaGraphExecDestroy(f->graph_exec);
   if (f->capture_stream) cudaStreamDestroy(f->capture_stream);
+  gr::count_object(f->device, -1);
   delete f;
   return GR_OK;
 }
@@ -567,9 +692,9 @@ gr_status gr_readback(gr_frame* f, int32_t view, float* dst, size_t dst_bytes, i
   for (int b = 0; b < s.nb; ++b) inv[b] = f->counts[view][b] > 0 ? 1.0f / (float)f->counts[view][b] : 0.0f;
   float* inv_d = nullptr;
   float* tmp = nullptr;
-  cudaError_t e = cudaMallocAsync(&inv_d, sizeof(float) * s.nb, st);
+  cudaError_t e = gr::dev_alloc(&inv_d, sizeof(float) * s.nb, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(inv_d, inv.data(), sizeof(float) * s.nb, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && !dst_is_device) e = cudaMallocAsync(&tmp, n * sizeof(float), st);
+  if (e == cudaSuccess && !dst_is_device) e = gr::dev_alloc(&tmp, n * sizeof(float), st);
   if (e == cudaSuccess) e = gr::readback_impl(f, view, dst_is_device ? dst : tmp, inv_d, st);
   if (e == cudaSuccess && !dst_is_device) e = cudaMemcpyAsync(dst, tmp, n * sizeof(float), cudaMemcpyDeviceToHost, st);
   if (inv_d) cudaFreeAsync(inv_d, st);

@@ -11,6 +11,14 @@
 
 namespace gr {
 
+// Device memory of the library's objects and calls, stream-ordered, from a pool
+// of the current device; freed with cudaFreeAsync (or cudaFree once idle).
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
+template <class T>
+cudaError_t dev_alloc(T** p, size_t bytes, cudaStream_t st) {
+  return dev_alloc((void**)p, bytes, st);
+}
+
 // The 16-bit grid of the default nodes' child boxes: coordinate = lo + q step.
 struct GridDesc {
   float lo[3], step[3];

@@ -742,7 +742,7 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
   const size_t o_box = take(sizeof(float) * 6 * 2 * N), o_id = take(sizeof(int) * 2 * N), o_p = take(sizeof(int) * N);
   const size_t o_sums = take(sizeof(int2) * (N / kTile + 1));
   unsigned char* d = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&d, off, st);
+  cudaError_t e = dev_alloc((void**)&d, off, st);
   if (e != cudaSuccess) return e;
   BuildState* S = (BuildState*)(d + o_state);
   float4* cen = (float4*)(d + o_cen);

@@ -1968,7 +1968,7 @@ __global__ void k_debug_rng(uint32_t seed, uint32_t view, uint32_t pixel, uint32
 cudaError_t debug_rng_impl(uint32_t seed, uint32_t view, uint32_t pixel, uint32_t sample, int seg, int call, int n,
                            uint32_t* host_out, cudaStream_t st) {
   uint4* d = nullptr;
-  cudaError_t e = cudaMallocAsync(&d, sizeof(uint4) * (size_t)n, st);
+  cudaError_t e = dev_alloc(&d, sizeof(uint4) * (size_t)n, st);
   if (e != cudaSuccess) return e;
   k_debug_rng<<<(n + 255) / 256, 256, 0, st>>>(seed, view, pixel, sample, seg, call, n, d);
   e = cudaGetLastError();
@@ -1990,7 +1990,7 @@ __global__ void k_debug_table(double x, int jmax, float* out) {
 cudaError_t debug_table_impl(float height_um, double lambda_um, int jmax, int dtype, float* host_out,
                              cudaStream_t st) {
   float* d = nullptr;
-  cudaError_t e = cudaMallocAsync(&d, sizeof(float) * (size_t)(jmax + 1), st);
+  cudaError_t e = dev_alloc(&d, sizeof(float) * (size_t)(jmax + 1), st);
   if (e != cudaSuccess) return e;
   const double x = kPiD * (double)height_um / lambda_um;  // pi h / lambda, as in k_tables
   const int grid = (jmax + 256) / 256;
@@ -2020,8 +2020,8 @@ __global__ void k_debug_footprint(int n, const float4* in, float2* out) {
 cudaError_t debug_footprint_impl(int n, const float* host_in, float* host_out, cudaStream_t st) {
   float4* din = nullptr;
   float2* dout = nullptr;
-  cudaError_t e = cudaMallocAsync(&din, sizeof(float4) * (size_t)n, st);
-  if (e == cudaSuccess) e = cudaMallocAsync(&dout, sizeof(float2) * (size_t)n, st);
+  cudaError_t e = dev_alloc(&din, sizeof(float4) * (size_t)n, st);
+  if (e == cudaSuccess) e = dev_alloc(&dout, sizeof(float2) * (size_t)n, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(din, host_in, sizeof(float4) * (size_t)n, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     k_debug_footprint<<<std::min((n + 255) / 256, 4096), 256, 0, st>>>(n, din, dout);
@@ -2336,7 +2336,7 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     if (f->scratch) cudaFreeAsync(f->scratch, st);
     f->scratch = nullptr;
     f->scratch_bytes = 0;
-    if (cudaMallocAsync(&f->scratch, total, st) != cudaSuccess) {
+    if (dev_alloc(&f->scratch, total, st) != cudaSuccess) {
       err = "scratch allocation failed";
       return GR_E_OOM;
     }
