@@ -101,6 +101,7 @@ struct RenderParams {
   int table_vals_count;
   Pool pool;
   int P;
+  int multi_sample;      // 1 if a view's tickets can have more than one sample (slot accumulators in use)
   int regen_thr;         // regeneration threshold, percent of idle slots (0 = always)
   Counters* ctr;
 };
