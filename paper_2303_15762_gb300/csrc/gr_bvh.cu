@@ -288,8 +288,12 @@ __device__ __forceinline__ void write_node(float* __restrict__ Nd, const Box6& a
 // scene creation 3.3 -> 1.24 ms (1.01M triangles: 23.9 -> 3.8).
 constexpr int kTile = 256, kTail = 1024;
 constexpr int kPairThreads = kTile + 32;  // the tile and the clusters on either side, a thread each
-// levels of the collapse enqueued at a time (a scene that takes more waits once more per batch)
-constexpr int kLevelBatch = 18;
+// Levels of the collapse enqueued at once: n triangles take 1.3 to 1.6 log4(n)
+// levels (2: 1, 1172: 8, 5k: 9 or 10, 37k: 12, 92k: 13, 280k: 13 or 14, 1.01M:
+// 16), an empty level costs its launch (~2.3 us; with 18 for every scene a
+// two-triangle one took 203 us to create, now 151), one too few another wait.
+inline int first_levels(int n) { return std::min(n - 1, (int)std::ceil(1.55 * std::log2((double)n) / 2.0) + 1); }
+constexpr int kMoreLevels = 8;
 
 // Nearest neighbours of a tile (and of the 8 clusters on either side, whose
 // choice decides who is mutual), the pairs that merge, and the tile's counts.
@@ -783,13 +787,14 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
       float* nbox = Bc;  // the cluster boxes and ids have served
       int* front = Cc;
       k_grid_steps<<<std::min(g256, 1024), 256, 0, st>>>(tri, nodes, n, S, parity, nbox, front);
-      int level = 0;
+      int level = 0, batch = first_levels(n);
       do {
-        for (int k = 0; k < kLevelBatch && level < kMaxLevels; ++k, ++level) {
+        for (int k = 0; k < batch && level < kMaxLevels; ++k, ++level) {
           const double widest = level < 14 ? std::pow(4.0, level) : 3e8;
           const int blocks = (int)((std::min(widest, (double)n) + 127) / 128);
           k_collapse<<<blocks, 128, 0, st>>>(nodes, nbox, tri, front, S, parity, level, wn, gn);
         }
+        batch = kMoreLevels;
         if ((r = cudaMemcpyAsync(&h, S, sizeof h, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return r;
         if ((r = cudaStreamSynchronize(st)) != cudaSuccess) return r;
       } while (h.m[parity] == 1 && h.level_count[level] > 0 && level < kMaxLevels);
