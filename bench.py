@@ -48,10 +48,13 @@ FLOP_PER_TRI = 41
 # a 4-wide quantised node: per child 6 slab FMAs + 11 min/max + 4 for widening
 # and compare (25), plus 9 for the node's affine decode (3 mul, 3 sub, 3 mul)
 FLOP_PER_WNODE = 109
+# a 4-wide grid node (the default tree): per child 6 slab FMAs, 6 min/max and a
+# compare (19), and 3 for the nearest of four
+FLOP_PER_GNODE = 79
 KERNELS = ["k_regen", "k_trace", "k_shade", "k_shadow"]
 # DRAM traffic of the dominant kernel per unit (ray) from one ncu capture:
 # dram__bytes_read.sum + dram__bytes_write.sum of the second k_trace launch of
-# the 256x256 x 64 spp case (162.50 + 7.37 MB), divided by the rays it traced
+# the 256x256 x 64 spp case (164.22 + 7.97 MB), divided by the rays it traced
 # (the full default pool: one slot per ticket, 2,097,152 slots, all live in
 # the second iteration, plus about a thousand next-event rays, not counted);
 # traffic grows with the rays a launch processes.  Valid only for the
@@ -864,7 +867,7 @@ def main():
         # triangle tests per query, counted on the oracle's crop), so that the
         # work does not depend on the GPU's own tree; the kernels' own counts
         # are reported beside it.
-        per_node = FLOP_PER_WNODE if args.wide else FLOP_PER_NODE
+        per_node = FLOP_PER_WNODE if args.wide else FLOP_PER_GNODE
         trav_ms = (kms[1] + kms[3]) / args.steps
         queries = (stats["segments"] + stats["shadow_rays"])
         flops_kernel = (visits * per_node + tests * FLOP_PER_TRI) / args.steps
@@ -885,7 +888,7 @@ def main():
                 "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
                 "frac": achieved / peak_tflops, "work_basis": basis,
                 "achieved_kernel_counts": achieved_kernel,
-                "kernel_counts": "%.2f node visits and %.2f triangle tests per query in the GPU's PLOC tree" % (
+                "kernel_counts": "%.2f node visits and %.2f triangle tests per query in the GPU's 4-wide PLOC tree" % (
                     visits / args.steps / max(queries, 1), tests / args.steps / max(queries, 1)),
                 "peak_source": "measured: FP32 FMA-chain microbenchmark, gr_measure_fp32_peak (best of 3, %.2f ms); "
                                "nominal 152 SM x 128 lanes x 2 FLOP x 2070 MHz = %.1f" % (peak_ms, FP32_PEAK_TFLOPS),
