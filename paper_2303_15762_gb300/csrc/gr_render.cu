@@ -27,6 +27,8 @@
 // one regen pass for its ray, so its fold still follows its last term.
 // All launches have fixed shapes (grid-stride loops over device-side queue
 // counts), so a batch of iterations can be replayed as one CUDA graph.
+// Scenes of a few triangles without next-event estimation take one launch per
+// render instead (k_paths): a thread owns a ticket, the path in registers.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -1544,6 +1546,12 @@ __global__ void __launch_bounds__(256, MODE == 1   ? GR_SHADE_MIN_BLOCKS_HERO
 // ~300 bytes of slot state per segment and iteration for two triangle tests.
 // Measured: a grating of two triangles, 64^2 x 64 spp, 1213 -> 212 us per
 // render; four progressive requests (3.3M paths) 1291 -> 400 us per frame.
+// The line at 16 triangles, one launch against the wavefront (us, 16 bins,
+// Stokes 4): at 64^2 x 16 spp, 4 segments 122 against 415 at 16 triangles, 172
+// against 453 at 32 and 757 against 500 at 256; at 512^2 x 16 spp 1187 against
+// 1392 at 16, 1624 against 1508 at 32; at 512^2 x 64 spp, 6 segments 3382
+// against 4411 at 16, 5575 against 5310 at 32.  Every triangle is tested, so the
+// large views lose from 32 on.
 #ifndef GR_PATHS_TRIS
 #define GR_PATHS_TRIS 16
 #endif
@@ -2523,7 +2531,9 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       cudaEventDestroy(pe[0]);
       cudaEventDestroy(pe[1]);
     }
-    if (e == cudaSuccess && o.use_graph) e = cudaStreamSynchronize(st);  // as the graph's launch: the call waits
+    // the call waits, as the wavefront's loop and the graph's launch do: a caller may use the
+    // accumulators on another stream, or capture is refused, as on those
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
       err = std::string("launch: ") + cudaGetErrorString(e);
       return GR_E_CUDA;
