@@ -60,7 +60,7 @@ KERNELS = ["k_regen", "k_trace", "k_shade", "k_shadow"]
 # traffic grows with the rays a launch processes.  Valid only for the
 # traversal sources whose hash (source_hash) is recorded with it (else
 # reported null).
-NCU_TRAFFIC_PER_RAY = {("k_trace", "374dc2e6c0ef425d"): (162.498816e6 + 7.366912e6) / 2097152}
+NCU_TRAFFIC_PER_RAY = {("k_trace", "815f7ec5e2dff266"): (164.217088e6 + 7.971328e6) / 2097152}
 # the glass workload: a constant environment of this radiance lets paths
 # refracted through the glass reach a light, and the oracle crop (x0, y0,
 # side) is where the glass decides the most pixel-bins of the 512^2 view

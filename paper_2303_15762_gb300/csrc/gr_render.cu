@@ -1545,7 +1545,8 @@ __global__ void __launch_bounds__(256, MODE == 1   ? GR_SHADE_MIN_BLOCKS_HERO
 // The wavefront is bound there by what it moves and launches: four kernels and
 // ~300 bytes of slot state per segment and iteration for two triangle tests.
 // Measured: a grating of two triangles, 64^2 x 64 spp, 1213 -> 212 us per
-// render; four progressive requests (3.3M paths) 1291 -> 400 us per frame.
+// render; four progressive requests (3.3M paths) 1291 -> 400 us per frame (the
+// host not waiting; the call waits: ~40 us more).
 // The line at 16 triangles, one launch against the wavefront (us, 16 bins,
 // Stokes 4): at 64^2 x 16 spp, 4 segments 122 against 415 at 16 triangles, 172
 // against 453 at 32 and 757 against 500 at 256; at 512^2 x 16 spp 1187 against
