@@ -24,8 +24,9 @@
  *     device pointers passed in are borrowed until the work enqueued on the
  *     given stream completes.
  *   - stream arguments are cudaStream_t values passed as void* (NULL = the
- *     legacy default stream); work is enqueued asynchronously and the caller
- *     synchronises on its own stream.
+ *     legacy default stream).  gr_frame_create, gr_frame_wrap and
+ *     gr_frame_reset enqueue and return; the other calls that take a stream
+ *     return when their work on it is done.
  *   - units: scene geometry in metres; optical lengths (wavelengths, grating
  *     period and height, roughness, correlation and coherence lengths, pixel
  *     pitch) in micrometres.
@@ -238,7 +239,8 @@ typedef struct {
  * Errors: GR_E_INVALID (null/negative sizes, material index out of range,
  * unknown material or light type), GR_E_OOM, GR_E_CUDA. */
 gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene** out);
-/* Free the scene.  Synchronises its device (a render may still read it).  The
+/* Free the scene.  Synchronises its device (another thread's render may still
+ * read it).  The
  * library keeps up to 256 MB of freed device memory for its next calls (512 MB
  * while scenes or frames live) and gives it back when an allocation fails. */
 gr_status gr_scene_destroy(gr_scene* scene);
@@ -282,9 +284,11 @@ gr_status gr_frame_reset(gr_frame* frame, void* cuda_stream);
  * the caller's).  Synchronises the device. */
 gr_status gr_frame_release(gr_frame* frame);
 
-/* Enqueue the samples [first_sample, first_sample + spp) of every view on the
+/* Render the samples [first_sample, first_sample + spp) of every view on the
  * stream, adding them into frame (which must have been created for views of
- * the same shapes).  Each sample is one path of Algorithm 1: a generalized
+ * the same shapes).  The call returns, with whatever status, when nothing of
+ * it is left running: the accumulators, the frame and its scratch may then be
+ * used on any stream.  Each sample is one path of Algorithm 1: a generalized
  * ray sourced from the pixel (Eq. MC_sourcing; Sec. 7.2: uniform position on
  * the pixel, rho = 0, beta = f_beta * p_pix_um, one wavelength bin), traced
  * through scenes[view.scene_index] with the footprint update of

@@ -305,7 +305,8 @@ def make_opts(seed=1, flags=0, table_dtype="f32", pool_size=0, block=0, use_grap
 
 
 def render(scenes, views, frame, stream=None, **opts):
-    """Enqueue the samples of every view into `frame` (asynchronous)."""
+    """Render the samples of every view into `frame`; returns when they are in
+    its accumulators, so any stream may use them."""
     L = lib_handle()
     sc = (ctypes.c_void_p * len(scenes))(*[s.handle.value for s in scenes])
     arr = pack_views(views)

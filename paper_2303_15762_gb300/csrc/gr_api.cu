@@ -451,8 +451,8 @@ gr_status gr_scene_bytes(const gr_scene* scene, size_t* bytes_out) {
 
 gr_status gr_scene_destroy(gr_scene* scene) {
   if (!scene) return fail(GR_E_INVALID, "gr_scene_destroy: null scene");
-  // a render may still read the scene (gr_render returns before its work is
-  // done): its memory goes back to the pool only after that
+  // another thread's render may still read the scene: its memory goes back to
+  // the pool only after that
   int dev = -1;
   const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != scene->device;
   if (other) cudaSetDevice(scene->device);

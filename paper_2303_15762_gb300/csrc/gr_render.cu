@@ -2469,9 +2469,13 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     e = (x);                                     \
     if (e != cudaSuccess) {                      \
       err = std::string(#x) + ": " + cudaGetErrorString(e); \
+      cudaStreamSynchronize(st);                 \
       return GR_E_CUDA;                          \
     }                                            \
   } while (0)
+  // From here on every exit waits for the stream: the next call on this frame,
+  // on whatever stream, resets the counters and the slots that this call's
+  // launches read, and may free its scratch.
   GR_CK(cudaMemcpyAsync(base + o_views, plan.views.data(), sizeof(DevView) * n_views, cudaMemcpyHostToDevice, st));
   GR_CK(cudaMemcpyAsync(base + o_vdesc, vd, sizeof(gr_view_desc) * n_views, cudaMemcpyHostToDevice, st));
   k_views<<<(n_views + 63) / 64, 64, 0, st>>>((const gr_view_desc*)(base + o_vdesc), (DevView*)(base + o_views), n_views);
@@ -2532,9 +2536,8 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       cudaEventDestroy(pe[0]);
       cudaEventDestroy(pe[1]);
     }
-    // the call waits, as the wavefront's loop and the graph's launch do: a caller may use the
-    // accumulators on another stream, or capture is refused, as on those
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const cudaError_t es = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) {
       err = std::string("launch: ") + cudaGetErrorString(e);
       return GR_E_CUDA;
@@ -2596,7 +2599,8 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
 
   // ---- iteration loop: batches of B iterations; the host watches the
   // device's live-slot count of the batch before the last one, so up to 2 B - 1
-  // iterations run past the end, ~13 us each.  At B = 8 / 4 / 2: 5.77 / 5.50 /
+  // iterations run past the end, ~13 us each, and the call returns when they
+  // are done.  At B = 8 / 4 / 2: 5.77 / 5.50 /
   // 5.41 ms (317 x 211 x 64 spp, anisotropic), 1.86 / 1.72 / 1.60 ms (256 x 192
   // x 16 spp); two iterations are still more device time than their launches
   // and the wait take on the host.
@@ -2656,6 +2660,7 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       if (e != cudaSuccess) {
         f->graph_exec = nullptr;
         err = std::string("render graph: ") + cudaGetErrorString(e);
+        cudaStreamSynchronize(st);
         return GR_E_CUDA;
       }
       f->graph_key = key;
@@ -2723,6 +2728,11 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       break;
     }
   }
+  e = cudaStreamSynchronize(st);  // the last batch and its counter copy
+  if (e != cudaSuccess && status == GR_OK) {
+    err = std::string("render: ") + cudaGetErrorString(e);
+    status = GR_E_CUDA;
+  }
   f->iterations += it;
   if (profile) {
     // per-kernel device time of this render
@@ -2730,7 +2740,6 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       f->kernel_ms[k] = 0.0;
       f->kernel_launches[k] = 0;
     }
-    if (status == GR_OK && !pev.empty()) cudaEventSynchronize(pev.back());
     // launch order regen, trace, shadow, shade; reported as 0 regen, 1 trace,
     // 2 shade, 3 shadow
     const int slot_of[4] = {0, 1, 3, 2};
