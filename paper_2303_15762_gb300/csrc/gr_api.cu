@@ -185,6 +185,19 @@ int current_device() {
   return d;
 }
 
+// The calling thread works on `dev` while this lives.
+struct OnDevice {
+  int before = -1;
+  bool other = false;
+  explicit OnDevice(int dev) {
+    other = cudaGetDevice(&before) == cudaSuccess && before != dev;
+    if (other) cudaSetDevice(dev);
+  }
+  ~OnDevice() {
+    if (other) cudaSetDevice(before);
+  }
+};
+
 // Frame over caller-owned accumulators (acc != nullptr, not zeroed: the
 // caller's buffer is added into) or library-owned ones (zeroed on stream).
 gr_status frame_make(const char* who, const gr_view_desc* views, int32_t n_views, float* acc, cudaStream_t st,
@@ -453,13 +466,10 @@ gr_status gr_scene_destroy(gr_scene* scene) {
   if (!scene) return fail(GR_E_INVALID, "gr_scene_destroy: null scene");
   // another thread's render may still read the scene: its memory goes back to
   // the pool only after that
-  int dev = -1;
-  const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != scene->device;
-  if (other) cudaSetDevice(scene->device);
+  const OnDevice on(scene->device);
   cudaDeviceSynchronize();
   if (scene->mem) cudaFree(scene->mem);
   gr::count_object(scene->device, -1);
-  if (other) cudaSetDevice(dev);
   delete scene;
   return GR_OK;
 }
@@ -513,6 +523,9 @@ gr_status gr_frame_reset(gr_frame* f, void* cuda_stream) {
 
 gr_status gr_frame_release(gr_frame* f) {
   if (!f) return fail(GR_E_INVALID, "gr_frame_release: null frame");
+  // the frame's own device, whichever is current: its memory and its pinned
+  // counters go to the next frame
+  const OnDevice on(f->device);
   cudaDeviceSynchronize();
   if (f->acc && f->owns_acc) cudaFree(f->acc);
   if (f->scratch) cudaFree(f->scratch);
