@@ -150,7 +150,9 @@ typedef struct {
  * GR_FLAG_FP32_NODES walks the binary tree with FP32 child boxes (64 bytes per
  * node); GR_FLAG_WIDE_BVH traverses the 4-wide tree with 8-bit child boxes
  * relative to each node, one ray per thread (all three give the same closest
- * hits: a box that contains the FP32 box is entered whenever the FP32 box is); GR_FLAG_HERO hero-wavelength spectral MIS (Sec. 7.2):
+ * hits: a box that contains the FP32 box is entered whenever the FP32 box is; a
+ * call with a scene whose tree is too deep for 4-wide nodes walks the FP32
+ * nodes); GR_FLAG_HERO hero-wavelength spectral MIS (Sec. 7.2):
  * with n_bins a multiple of 4, a path's bin is the hero of the class of bins
  * {c, c+Q, c+2Q, c+3Q} (Q = n_bins/4) and drives every sampling decision;
  * every connection to a light (escape, emitter hit, next-event estimate) is

@@ -723,8 +723,9 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
 // Build the trees of `n` triangles (device arrays verts [n][9], tri_mat [n]).
 // Outputs (device, caller-allocated): tri [n][3] float4, tmat [n], nodes
 // [(n-1)][16] floats, keys [n], and the 4-wide nodes wn and gn of up to n - 1
-// nodes each; on the host *n_wide (their count), *grid (the grid of gn's
-// boxes) and *grid_ok (whether it serves the scene).  One scratch allocation;
+// nodes each; on the host *n_wide (their count, 0 if n < 2 or the tree is too
+// deep for them), *grid (the grid of gn's boxes) and *grid_ok (whether it
+// serves the scene).  One scratch allocation;
 // the host waits once, for the state the launches leave behind, and again only
 // if the clustering or the collapse takes more rounds than were enqueued.
 cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* tri, int* tmat, float* nodes,
@@ -799,7 +800,10 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
         if ((r = cudaStreamSynchronize(st)) != cudaSuccess) return r;
       } while (h.m[parity] == 1 && h.level_count[level] > 0 && level < kMaxLevels);
       if (h.m[parity] == 1) {
-        if (h.created[parity] != n - 1 || h.level_count[level] > 0) return cudaErrorUnknown;
+        if (h.created[parity] != n - 1) return cudaErrorUnknown;
+        // a tree of more than kMaxLevels wide levels (equal boxes merge into a
+        // chain: 770 triangles on one another) keeps its binary nodes only
+        if (h.level_count[level] > 0) return cudaGetLastError();
         *n_wide = h.level_first[level];
         *grid = h.g;
         *grid_ok = !h.bad && (long long)h.small * 16 <= n;

@@ -2184,14 +2184,15 @@ const void* trace_kernel(int tree) {
                            : tree == kTreeGrid ? (const void*)k_trace<kTreeGrid> : (const void*)k_trace<kTreeF32>;
 }
 // The tree a render walks: the 8-bit 4-wide one on request, else the 4-wide
-// nodes on the 16-bit grid unless FP32 nodes are requested or a scene has no
-// grid nodes (GridState; scenes of fewer than 2 triangles need no nodes).
+// nodes on the 16-bit grid unless FP32 nodes are requested; the FP32 nodes if a
+// scene has not the ones wanted (build_trees; scenes of fewer than 2 triangles
+// need no nodes).
 int pick_tree(int flags, gr_scene* const* scenes, int n_scenes) {
-  if (flags & GR_FLAG_WIDE_BVH) return kTreeWide;
-  if (flags & GR_FLAG_FP32_NODES) return kTreeF32;
+  if (flags & GR_FLAG_FP32_NODES && !(flags & GR_FLAG_WIDE_BVH)) return kTreeF32;
   for (int i = 0; i < n_scenes; ++i)
-    if (scenes[i]->n_tris >= 2 && !scenes[i]->dev.gnodes) return kTreeF32;
-  return kTreeGrid;
+    if (scenes[i]->n_tris >= 2 && (flags & GR_FLAG_WIDE_BVH ? scenes[i]->dev.n_wide == 0 : !scenes[i]->dev.gnodes))
+      return kTreeF32;
+  return flags & GR_FLAG_WIDE_BVH ? kTreeWide : kTreeGrid;
 }
 // Whether a render takes the one-launch form (k_paths): the plain mode without
 // next-event estimation, no iteration bound asked for, and no view's scene of
