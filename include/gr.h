@@ -145,7 +145,7 @@ typedef struct {
  * propagating orders); the default tree is the binary BVH collapsed
  * into nodes of up to four children, with child boxes on a 16-bit grid over
  * the scene's bounds, rounded outward (64 bytes per node; a call with a scene
- * that has a coordinate beyond 1e12, or more than one in 16 of whose triangles
+ * that has a coordinate beyond 1e12, a tree too deep, or more than one in 16 of whose triangles
  * is smaller than 8 steps of its grid, walks the FP32 nodes instead);
  * GR_FLAG_FP32_NODES walks the binary tree with FP32 child boxes (64 bytes per
  * node); GR_FLAG_WIDE_BVH traverses the 4-wide tree with 8-bit child boxes

@@ -48,6 +48,7 @@ struct BuildState {
   int clo[3], chi[3];   // centroid bounds as ordered integers
   int lo[3], hi[3];     // vertex bounds as ordered integers
   int bad, small;       // coordinates out of the grid's range; triangles smaller than 8 grid steps
+  int deep;             // a walk of the 4-wide grid nodes could need more than kGridStackDepth entries
   GridDesc g;
   int m[2], created[2]; // clusters left and nodes created, by parity of the round
   int tiles_done;       // tiles of the round that have counted their pairs
@@ -60,7 +61,7 @@ __global__ void k_build_init(BuildState* B, int n) {
     B->chi[t] = B->hi[t] = (int)0x80000000;
   }
   if (t == 0) {
-    B->bad = B->small = B->tiles_done = 0;
+    B->bad = B->small = B->deep = B->tiles_done = 0;
     B->m[0] = n;
     B->created[0] = 0;
   }
@@ -556,14 +557,15 @@ __device__ __forceinline__ float half_area(const BoxF& b) {
 }
 
 // The 16-bit grid of a scene: its bounds in 65535 steps per axis.  It serves
-// unless a coordinate is not finite or beyond 1e12, or it is so coarse against
+// unless a coordinate is not finite or beyond 1e12, a walk of the tree could
+// need more than the kGridStackDepth entries it has, or it is so coarse against
 // the triangles (more than one in 16 smaller than 8 steps) that their boxes
 // would swell; the renders of such a scene walk the FP32 nodes.  The same
 // launch stores the box of every binary internal node (from its parent's
 // child boxes).
 __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ tri, const float* __restrict__ nodes, int n,
                                                     BuildState* S, int parity, float* __restrict__ nbox,
-                                                    int* __restrict__ front) {
+                                                    int* __restrict__ front, int* __restrict__ pend) {
   if (S->m[parity] != 1) return;  // the clustering needs more rounds
   GridDesc g;
   float widest = 0.0f;
@@ -575,6 +577,7 @@ __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ t
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     S->g = g;
     front[0] = 0;  // wide node 0 stands for the root
+    pend[0] = 0;
   }
   int small = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -600,11 +603,14 @@ __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ t
 }
 
 // One level of the top-down collapse.  front[w] is the binary node that wide
-// node w stands for; level L's nodes are [level_first[L], + level_count[L]),
+// node w stands for, pend[w] the most entries a walk that enters w can have on
+// its stack: every node on the way pushed its internal children but the one
+// walked next.  (A bound by levels would not do: the way to w may have taken a
+// wide level for each binary one, with three entries left at each.)  Level L's nodes are [level_first[L], + level_count[L]),
 // and a node's internal children take consecutive places in the next level.
 __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ nodes, const float* __restrict__ nbox,
                                                   const float4* __restrict__ tri, int* __restrict__ front,
-                                                  BuildState* S, int parity, int level, uint4* __restrict__ wn,
+                                                  int* __restrict__ pend, BuildState* S, int parity, int level, uint4* __restrict__ wn,
                                                   uint4* __restrict__ gn) {
   if (S->m[parity] != 1) return;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -670,12 +676,15 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
   int refs[4] = {-1, -1, -1, -1};
   int inner = 0;
   for (int c = 0; c < cnt; ++c) inner += ch[c] >= 0;
+  const int below = pend[widx] + max(inner - 1, 0);
+  if (below > kGridStackDepth) S->deep = 1;
   int w = inner ? first + count + atomicAdd(&S->level_count[level + 1], inner) : 0;
   for (int c = 0; c < cnt; ++c) {
     if (ch[c] < 0) {
       refs[c] = ch[c];
     } else {
       refs[c] = w;
+      pend[w] = below;
       front[w++] = ch[c];
     }
   }
@@ -785,15 +794,15 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
       k_ploc_tail<<<1, kTail, 0, st>>>(Bc, Cc, S, parity, n, nodes);
       // the collapse is enqueued with the rounds; its launches return at once
       // if the clustering is not done, and are enqueued again after the next ones
-      float* nbox = Bc;  // the cluster boxes and ids have served
-      int* front = Cc;
-      k_grid_steps<<<std::min(g256, 1024), 256, 0, st>>>(tri, nodes, n, S, parity, nbox, front);
+      float* nbox = Bc;  // the cluster boxes, ids and pairs have served
+      int *front = Cc, *pend = P;
+      k_grid_steps<<<std::min(g256, 1024), 256, 0, st>>>(tri, nodes, n, S, parity, nbox, front, pend);
       int level = 0, batch = first_levels(n);
       do {
         for (int k = 0; k < batch && level < kMaxLevels; ++k, ++level) {
           const double widest = level < 14 ? std::pow(4.0, level) : 3e8;
           const int blocks = (int)((std::min(widest, (double)n) + 127) / 128);
-          k_collapse<<<blocks, 128, 0, st>>>(nodes, nbox, tri, front, S, parity, level, wn, gn);
+          k_collapse<<<blocks, 128, 0, st>>>(nodes, nbox, tri, front, pend, S, parity, level, wn, gn);
         }
         batch = kMoreLevels;
         if ((r = cudaMemcpyAsync(&h, S, sizeof h, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return r;
@@ -806,7 +815,7 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
         if (h.level_count[level] > 0) return cudaGetLastError();
         *n_wide = h.level_first[level];
         *grid = h.g;
-        *grid_ok = !h.bad && (long long)h.small * 16 <= n;
+        *grid_ok = !h.bad && !h.deep && (long long)h.small * 16 <= n;
         return cudaGetLastError();
       }
       if (rounds == 0 || h.m[parity] >= bound) break;  // no pair merges (boxes that are not finite)

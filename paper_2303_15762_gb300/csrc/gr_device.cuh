@@ -21,7 +21,9 @@ constexpr float kGCont = 50.0f;
 // Largest grating order magnitude kept in the order tables.
 constexpr int kMaxOrder = 40;
 constexpr int kStackDepth = 64;
-// the 4-wide walk pushes up to three children per two binary levels
+// The 4-wide walk pushes up to three children per level.  A scene whose tree
+// could need more entries has no grid nodes (k_collapse counts them; procedural
+// scenes of 8k, 16k and 124k triangles need 25, 27 and 33).
 constexpr int kGridStackDepth = 96;
 // BVH layouts a traversal can walk: the binary tree with FP32 child boxes (64
 // bytes per node), its collapse into nodes of up to four children with child

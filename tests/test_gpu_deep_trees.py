@@ -1,7 +1,9 @@
 """Scenes whose trees are chains: triangles on one another merge one pair per
 round of the clustering, so n of them make n - 1 binary levels and a third as
 many 4-wide ones (256 at 769 triangles, 257 at 770).  They are created and
-render as any other scene, alone and inside one, whichever nodes are asked for."""
+render as any other scene, alone and inside one, whichever nodes are asked for.
+And scenes of nested shells, whose walk leaves three subtrees waiting at every
+level: 121 entries, where the binary tree's walk leaves 42."""
 import numpy as np
 import pytest
 
@@ -38,3 +40,24 @@ def test_equal_triangles(gr, oracle, n, inside):
         assert np.array_equal(a, gr.render_image(scene, v, seed=5, flags=gr.FLAG_NEE | flag))
     ref = oracle.Scene(scene).render(v, 5, gr.FLAG_NEE)
     assert_parity(a, ref)
+
+
+def test_nested_shells(gr):
+    """Seen from their common centre: 40 shells of 8 triangles, each 0.35 of the
+    last, whose boxes a ray along the axis enters and whose triangles it passes
+    (the smallest first: of boxes entered at once the walk takes the first)."""
+    t = []
+    for i in reversed(range(40)):
+        for j in range(8):
+            z = 0.35 ** i * (1 + 0.02 * j)
+            t.append([(-0.08 * z, 0.4 * z, z), (0.4 * z, -0.08 * z, z), (0.4 * z, 0.4 * z, z)])
+    ground = sg._tile_tris(np.array([0.0, -3.0, 0.0]), 4.0, 60, 0.1, np.random.default_rng(0), 0.0)
+    mats = [sg.material(sg.MAT_MIRROR, fresnel=1, n_re=0.4, n_im=3.0),
+            sg.material(sg.MAT_ROUGH, fresnel=1, n_re=0.3, n_im=3.5, sigma_h_um=0.2, corr_len_um=3.0)]
+    scene = sg._scene(np.concatenate([np.asarray(t), ground]), [0] * len(t) + [1] * len(ground), mats,
+                      [sg.light(sg.LIGHT_ENV, E=0.3)])
+    v = sg.view(eye=(0, 0, 0), look_at=(0, 0, 1.0), up=(0, 1, 0), vfov_deg=50.0, width=33, height=31, n_bins=2, spp=4,
+                max_depth=3)
+    a = gr.render_image(scene, v, seed=5, flags=gr.FLAG_NEE)
+    assert len(np.unique(a)) > 1
+    assert np.array_equal(a, gr.render_image(scene, v, seed=5, flags=gr.FLAG_NEE | gr.FLAG_FP32_NODES))
