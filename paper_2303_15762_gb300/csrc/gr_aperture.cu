@@ -86,7 +86,10 @@ __device__ __forceinline__ float cos_ftz(float x) {
 // Adds w e^-u2 cis(phase) of one sample to the sums of two directions; `in`:
 // the sample lies inside that direction's truncation radius.  The phase is
 // reduced to [-pi, pi], where the hardware sine and cosine have an absolute
-// error of ~1e-6, below the ~6e-5 rad to which the FP32 phase is known.
+// error of ~1e-6, below the ~6e-5 rad to which the FP32 phase is known.  FAR:
+// the phase of a sample outside the radius may be infinite or not a number,
+// and must not reach the sums through 0 x NaN.
+template <bool FAR>
 __device__ __forceinline__ void add_sample(float w, f32x2 u2, f32x2 phase, bool in0, bool in1, f32x2& re, f32x2& im) {
   const f32x2 mag = add2(mul2(phase, dup2(kInvTwoPi)), dup2(kRound));
   const f32x2 neg_n = fma2(mag, dup2(-1.0f), dup2(kRound));
@@ -94,6 +97,10 @@ __device__ __forceinline__ void add_sample(float w, f32x2 u2, f32x2 phase, bool 
   float e0, e1, r0, r1;
   unpack2(mul2(u2, dup2(kNegLog2e)), e0, e1);
   unpack2(r, r0, r1);
+  if (FAR) {
+    r0 = in0 ? r0 : 0.0f;
+    r1 = in1 ? r1 : 0.0f;
+  }
   const f32x2 g = pack2(in0 ? w * ex2_ftz(e0) : 0.0f, in1 ? w * ex2_ftz(e1) : 0.0f);
   re = fma2(g, pack2(cos_ftz(r0), cos_ftz(r1)), re);
   im = fma2(g, pack2(sin_ftz(r0), sin_ftz(r1)), im);
@@ -130,6 +137,7 @@ constexpr float kSkipSlack = 0.9999f;
 // Aperture samples in shared memory as (x, w); then the interval of each
 // chunk and the interval of all samples.  rot1, rot: cosine and sine of the
 // step to the lane's second direction and to its next pair.
+template <bool FAR>
 __global__ void __launch_bounds__(kApertureThreads, 7)
     k_aperture_backward(int n_split, const double* __restrict__ x0s, int n_ap, const float2* __restrict__ ap,
                         double beta, double z, double k, double reach, double dtheta, double rho_cut, double2 rot1,
@@ -204,7 +212,7 @@ __global__ void __launch_bounds__(kApertureThreads, 7)
         float u0, u1;
         unpack2(u, u0, u1);
         const f32x2 u2 = mul2(mul2(u, u), inv2);
-        add_sample(v.y, u2, fma2(kap2, dx, mul2(nrho2, u2)), !(fabsf(u0) > cut[0]), !(fabsf(u1) > cut[1]), re, im);
+        add_sample<FAR>(v.y, u2, fma2(kap2, dx, mul2(nrho2, u2)), !(fabsf(u0) > cut[0]), !(fabsf(u1) > cut[1]), re, im);
       }
     }
     float r[2], m[2];
@@ -226,6 +234,7 @@ __global__ void __launch_bounds__(kApertureThreads, 7)
 // sum_t |A|^2 s_z / (pi beta'^2) k^2 s_z^4 dt^2 / (2 pi)^2.  Aperture samples
 // are (x, y, weight, 0) in shared memory, then the chunks' boxes (x lo, x hi,
 // y lo, y hi) and the box of all samples.
+template <bool FAR>
 __global__ void __launch_bounds__(kApertureThreads, 5)
     k_aperture_backward_3d(int n_split, const double2* __restrict__ x0s, int n_ap, const float4* __restrict__ ap,
                            double beta, double z, double k, double reach, double dt, double rho_cut, int n_t,
@@ -295,7 +304,7 @@ __global__ void __launch_bounds__(kApertureThreads, 5)
         float p0, p1;
         unpack2(p2, p0, p1);
         const f32x2 u2 = mul2(p2, inv2);
-        add_sample(v.z, u2, fma2(nrho2, u2, fma2(kx2, dx, mul2(ky2, dy))), !(p0 > cut2[0]), !(p1 > cut2[1]), re, im);
+        add_sample<FAR>(v.z, u2, fma2(nrho2, u2, fma2(kx2, dx, mul2(ky2, dy))), !(p0 > cut2[0]), !(p1 > cut2[1]), re, im);
       }
     }
     float r[2], m[2];
@@ -412,6 +421,24 @@ cudaError_t run_aperture(int dim, const void* kernel, int n_det, const double* x
   return e;
 }
 
+// Whether a sample's phase in some direction may not be finite, so that the
+// kernels must mask it (FAR, two more selects per sample): D bounds the distance of
+// a sample from a landing point per axis, tan2 the directions' squared tangent.
+// The bounds are far above what the kernels form, and what is not a number
+// fails them.
+constexpr double kPhaseMax = 1e36;
+bool phases_far(double D, double tan2, double beta, double z, double k) {
+  const double ib = 1.0 / (beta * beta), q = 1.0 + tan2, d2 = 4.0 * D * D;
+  return !(k * D < kPhaseMax && q * d2 < kPhaseMax && d2 * ib < kPhaseMax &&
+           d2 * ib * (z / k) * ib * q < kPhaseMax);
+}
+// The largest magnitude of n values (infinity if one is not a number).
+double max_abs(const double* v, size_t n) {
+  double m = 0.0;
+  for (size_t i = 0; i < n; ++i) m = std::fabs(v[i]) <= m ? m : v[i] == v[i] ? std::fabs(v[i]) : INFINITY;
+  return m;
+}
+
 }  // namespace
 
 cudaError_t aperture_backward_3d_impl(int n_det, const double* x0_host, int n_ap, const double* xa_host,
@@ -419,11 +446,14 @@ cudaError_t aperture_backward_3d_impl(int n_det, const double* x0_host, int n_ap
                                       double dt, double rho_cut, double* out_host, cudaStream_t st, float* ms) {
   const int n_t = (int)std::ceil(2.0 * reach / (z * dt));  // at most 2^13 (checked at the entry)
   const double pi = 3.14159265358979323846;
-  return run_aperture(2, (const void*)k_aperture_backward_3d, n_det, x0_host, n_ap, xa_host, wa_host,
-                      (double)n_t * n_t, 1.0 / (4.0 * pi * pi), out_host, st, ms,
+  const double t = (max_abs(x0_host, 2 * (size_t)n_det) + reach) / z;
+  const bool far = phases_far(max_abs(xa_host, 2 * (size_t)n_ap) + reach, 2.0 * t * t, beta, z, k);
+  const auto kernel = far ? k_aperture_backward_3d<true> : k_aperture_backward_3d<false>;
+  return run_aperture(2, (const void*)kernel, n_det, x0_host, n_ap, xa_host, wa_host, (double)n_t * n_t,
+                      1.0 / (4.0 * pi * pi), out_host, st, ms,
                       [&](unsigned grid, int n_split, size_t smem, const void* x0, const void* ap, double* part) {
-                        k_aperture_backward_3d<<<grid, kApertureThreads, smem, st>>>(
-                            n_split, (const double2*)x0, n_ap, (const float4*)ap, beta, z, k, reach, dt, rho_cut, n_t, part);
+                        kernel<<<grid, kApertureThreads, smem, st>>>(n_split, (const double2*)x0, n_ap, (const float4*)ap,
+                                                                     beta, z, k, reach, dt, rho_cut, n_t, part);
                       });
 }
 
@@ -431,11 +461,14 @@ cudaError_t aperture_backward_impl(int n_det, const double* x0_host, int n_ap, c
                                    const double* wa_host, double beta, double z, double k, double reach,
                                    double dtheta, double rho_cut, double* out_host, cudaStream_t st, float* ms) {
   const double pi = 3.14159265358979323846;
-  return run_aperture(1, (const void*)k_aperture_backward, n_det, x0_host, n_ap, xa_host, wa_host,
+  const double t = (max_abs(x0_host, (size_t)n_det) + reach) / z;
+  const bool far = phases_far(max_abs(xa_host, (size_t)n_ap) + reach, t * t, beta, z, k);
+  const auto kernel = far ? k_aperture_backward<true> : k_aperture_backward<false>;
+  return run_aperture(1, (const void*)kernel, n_det, x0_host, n_ap, xa_host, wa_host,
                       2.0 * std::atan(reach / z) / dtheta + 1.0, 1.0 / (2.0 * pi), out_host, st, ms,
                       [&](unsigned grid, int n_split, size_t smem, const void* x0, const void* ap, double* part) {
                         const double step = 2.0 * kApertureThreads * n_split * dtheta;
-                        k_aperture_backward<<<grid, kApertureThreads, smem, st>>>(
+                        kernel<<<grid, kApertureThreads, smem, st>>>(
                             n_split, (const double*)x0, n_ap, (const float2*)ap, beta, z, k, reach, dtheta, rho_cut,
                             make_double2(std::cos(dtheta), std::sin(dtheta)),
                             make_double2(std::cos(step), std::sin(step)), part);
