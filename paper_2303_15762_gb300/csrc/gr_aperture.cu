@@ -23,13 +23,17 @@
 // unit, and samples are skipped 64 at a time when their interval or box lies
 // outside the truncation radius of all 64 directions of a warp.  The terms of
 // a direction are formed in FP64, of which the chip does 1/64 of the FP32
-// rate: sine and cosine come from the previous direction's by rotation, and
-// reciprocals and square roots from an FP32 seed and one Newton step (relative
-// error ~1e-14), ~25 FP64 operations per direction instead of several hundred.
+// rate: sine and cosine come from the previous direction's by rotation (at most
+// kApertureRotations in a row), and reciprocals and square roots from an FP32
+// seed and Newton steps, ~30 FP64 operations per direction instead of several
+// hundred.
 // Measured (kernel time, before -> after): double slit, 4001 elements x ~8900
 // directions x 800 samples 12.74 -> 4.66 ms; 13 elements 1192 -> 73 us (13
 // blocks before, 455 now); disk of 1152 samples, 400 elements x 61,009
-// directions 30.9 -> 18.9 ms (FMA pipe 67% busy, issue slots 70%).  One
+// directions 30.9 -> 18.9 ms (FMA pipe 67% busy, issue slots 70%).  The second
+// Newton steps cost 4.63 -> 4.64 ms there, and where FP64 weighs most, 5000
+// elements x 445,000 directions x 4 samples, 129 -> 161 ms (547 with FP64
+// divisions, roots and sines).  One
 // direction per lane with two samples packed took 4.9 and 17.8 ms, but sums
 // the samples in another order; sine and cosine as polynomials on the FMA pipe
 // 6.3 and 22.2 ms.
@@ -55,6 +59,12 @@ constexpr int kApertureChunk = 64;  // samples with one bounding box
 // weighs more)
 constexpr int kApertureBlocksPerSM = 32;
 
+// groups of directions a lane walks by rotation: each adds up to an FP64
+// rounding to sine and cosine, so an element of more directions takes more
+// blocks (up to kApertureBlocks of them in all)
+constexpr long long kApertureRotations = 256;
+constexpr long long kApertureBlocks = 1 << 24;
+
 // 2 pi split as hi + lo with hi the nearest float (Cody & Waite's additive
 // range reduction): x - n (2 pi) is formed as (x - n hi) - n lo with one
 // rounding per step, accurate to a few 1e-7 rad for |x| up to ~1e4.
@@ -68,7 +78,7 @@ constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an int
 // exponential without .ftz spends three more instructions on results below
 // 2^-126, which lie beyond sqrt(2 ln 2^126) = 13.2 widths: a truncation radius
 // beyond kFlushRadius takes it (FAR, which also masks phases; 1001 elements x
-// ~8900 directions x 800 samples, every sample inside: 4.26 -> 5.17 ms).
+// ~8900 directions x 800 samples, every sample inside: 4.26 -> 5.07 ms).
 constexpr double kFlushRadius = 13.0;
 template <bool FAR>
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -111,15 +121,13 @@ __device__ __forceinline__ void add_sample(float w, f32x2 u2, f32x2 phase, bool 
   im = fma2(g, pack2(sin_ftz(r0), sin_ftz(r1)), im);
 }
 
-// 1 / a and 1 / sqrt(a) of a positive normal a: FP32 seed, one Newton step in FP64.
-__device__ __forceinline__ double rcp_d(double a) {
-  const double r = (double)__frcp_rn((float)a);
-  return fma(r, fma(-a, r, 1.0), r);
-}
-__device__ __forceinline__ double rsqrt_d(double a) {
-  const double r = (double)__frsqrt_rn((float)a);
-  return fma(0.5 * r, fma(-a * r, r, 1.0), r);
-}
+// 1 / a and 1 / sqrt(a) of a positive normal a: FP32 seed, one Newton step in
+// FP64 (relative error ~1e-14, for what is rounded to FP32 next), and a second
+// one to FP64's own accuracy (for the FP64 weights).
+__device__ __forceinline__ double rcp_step(double a, double r) { return fma(r, fma(-a, r, 1.0), r); }
+__device__ __forceinline__ double rsqrt_step(double a, double r) { return fma(0.5 * r, fma(-a * r, r, 1.0), r); }
+__device__ __forceinline__ double rcp_d(double a) { return rcp_step(a, (double)__frcp_rn((float)a)); }
+__device__ __forceinline__ double rsqrt_d(double a) { return rsqrt_step(a, (double)__frsqrt_rn((float)a)); }
 
 // Block sum in a fixed order (warp shuffles, then the warps in turn).
 __device__ __forceinline__ void block_partial(double acc, double* out) {
@@ -178,7 +186,7 @@ __global__ void __launch_bounds__(kApertureThreads, 7)
     double s1 = sn, c1 = c;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const double r = rcp_d(c1);
+      const double r = rcp_step(c1, rcp_d(c1));
       const double t = zk * r;               // oblique path length over |k|
       const double rho = t * ib;             // Eq. K_free_space_propagation from rho = 0
       const double b2 = fma(rho, t, beta2);
@@ -189,7 +197,7 @@ __global__ void __launch_bounds__(kApertureThreads, 7)
       inv2b2[j] = (float)(0.5 * y * y);
       nrho[j] = -(float)rho;
       cut[j] = (float)(rho_cut * (b2 * y));
-      wgt[j] = c1 * c1 * wk * y;             // cos(theta) (pi b'^2)^(-1/2) dkappa
+      wgt[j] = c1 * c1 * wk * rsqrt_step(b2, y);  // cos(theta) (pi b'^2)^(-1/2) dkappa
       out[j] = i + j >= n_th || kSkipSlack * cf[j] * gap(xcf[j], all.x, all.y) > cut[j];
       if (j == 0) {
         s1 = fma(sn, rot1.x, c * rot1.y);
@@ -282,7 +290,8 @@ __global__ void __launch_bounds__(kApertureThreads, 5)
       inv2b2[j] = (float)(0.5 * ib2);
       nrho[j] = -(float)(zk * ib * q2 * sz);
       cut2[j] = (float)(rc2 * b2);
-      wgt[j] = s2 * s2 * sz * ib2 * wk;
+      const double szw = rsqrt_step(q2, sz), szw2 = szw * szw;
+      wgt[j] = szw2 * szw2 * szw * rcp_step(b2, ib2) * wk;
       gz[j] = kSkipSlack * -nsz2[j];  // |P d|^2 >= s_z^2 |d|^2
       const float hx = gap(cx[j], all.x, all.y), hy = gap(cy[j], all.z, all.w);
       out[j] = i + j >= n_dir || gz[j] * fmaf(hx, hx, hy * hy) > cut2[j];
@@ -333,11 +342,13 @@ __global__ void k_reduce(int n_det, int n_split, const double* __restrict__ part
 }
 
 // Blocks per detector element of at most n_dir directions: as many as it takes
-// to give the chip kApertureBlocksPerSM blocks per SM, each with the same
-// number of groups of directions.
+// to give the chip kApertureBlocksPerSM blocks per SM and a lane at most
+// kApertureRotations groups of directions, each block the same number of them.
 int split_of(long long n_det, double n_dir, int sms) {
   const long long groups = std::max(1LL, (long long)std::ceil(n_dir / (2 * kApertureThreads)));
-  const long long want = std::min(groups, ((long long)kApertureBlocksPerSM * sms + n_det - 1) / n_det);
+  const long long fill = ((long long)kApertureBlocksPerSM * sms + n_det - 1) / n_det;
+  const long long rotations = std::min((groups + kApertureRotations - 1) / kApertureRotations, kApertureBlocks / n_det);
+  const long long want = std::min(groups, std::max(fill, rotations));
   const long long per = (groups + want - 1) / want;
   return (int)((groups + per - 1) / per);
 }
