@@ -1242,6 +1242,15 @@ struct RcpTable {
 };
 __constant__ RcpTable c_rcp = RcpTable();
 
+// g / m from the rounded reciprocal r of m: the product corrected by its exact
+// remainder is the correctly rounded quotient (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
+// Dev. 1990), in three operations beside the serial product of the terms.
+__device__ __forceinline__ double quotient(double g, double m, double r) {
+  const double q = g * r;
+  return fma(fma(-q, m, g), r, q);
+}
+
 // Rough-surface term count m ~ Poisson(g), g = (2 k sigma_h cos_i)^2: the
 // first m whose cumulative Poisson probability exceeds u (at most 1000).
 __device__ __noinline__ int poisson_pick_fp64(double lam_d, float sigma_h_um, float cos_i, float u) {
@@ -1252,7 +1261,7 @@ __device__ __noinline__ int poisson_pick_fp64(double lam_d, float sigma_h_um, fl
   int mi = 0;
   while ((double)u >= cd && mi < 1000) {
     ++mi;
-    pd *= mi < 128 ? gd * c_rcp.r[mi] : gd / mi;  // no FP64 division in the serial chain
+    pd *= mi < 128 ? quotient(gd, (double)mi, c_rcp.r[mi]) : gd / mi;
     cd += pd;
   }
   return mi;
