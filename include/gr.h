@@ -26,7 +26,7 @@
  *   - stream arguments are cudaStream_t values passed as void* (NULL = the
  *     legacy default stream).  gr_frame_create, gr_frame_wrap and
  *     gr_frame_reset enqueue and return; the other calls that take a stream
- *     return when their work on it is done.
+ *     return when their results are complete.
  *   - units: scene geometry in metres; optical lengths (wavelengths, grating
  *     period and height, roughness, correlation and coherence lengths, pixel
  *     pitch) in micrometres.
@@ -288,9 +288,10 @@ gr_status gr_frame_release(gr_frame* frame);
 
 /* Render the samples [first_sample, first_sample + spp) of every view on the
  * stream, adding them into frame (which must have been created for views of
- * the same shapes).  The call returns, with whatever status, when nothing of
- * it is left running: the accumulators, the frame and its scratch may then be
- * used on any stream.  Each sample is one path of Algorithm 1: a generalized
+ * the same shapes).  The call returns when the samples are in the accumulators,
+ * which any stream may then use; what it still runs then finds nothing to do,
+ * and the library orders it before the next use of the frame's scratch and
+ * counters, whatever the stream.  Each sample is one path of Algorithm 1: a generalized
  * ray sourced from the pixel (Eq. MC_sourcing; Sec. 7.2: uniform position on
  * the pixel, rho = 0, beta = f_beta * p_pix_um, one wavelength bin), traced
  * through scenes[view.scene_index] with the footprint update of

@@ -531,6 +531,8 @@ gr_status gr_frame_release(gr_frame* f) {
   if (f->scratch) cudaFree(f->scratch);
   if (f->ctr) cudaFree(f->ctr);
   if (f->ctr_host) gr::unpin_counters(f->ctr_host);
+  for (cudaEvent_t ev : f->ev)
+    if (ev) cudaEventDestroy(ev);
   if (f->graph_exec) cudaGraphExecDestroy(f->graph_exec);
   if (f->capture_stream) cudaStreamDestroy(f->capture_stream);
   gr::count_object(f->device, -1);
@@ -721,7 +723,8 @@ gr_status gr_frame_stats(gr_frame* f, void* cuda_stream, gr_stats* out) {
   if (!f || !out) return fail(GR_E_INVALID, "gr_frame_stats: null argument");
   cudaStream_t st = (cudaStream_t)cuda_stream;
   gr::Counters c;
-  cudaError_t e = cudaMemcpyAsync(&c, f->ctr, sizeof c, cudaMemcpyDeviceToHost, st);
+  cudaError_t e = f->tail ? cudaStreamWaitEvent(st, f->tail, 0) : cudaSuccess;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&c, f->ctr, sizeof c, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "gr_frame_stats");
   out->samples = (int64_t)c.samples;

@@ -154,6 +154,11 @@ struct gr_frame {
   gr::Counters* ctr_host = nullptr;      // pinned mirror
   long long launches = 0;
   long long iterations = 0;
+  cudaEvent_t ev[2] = {nullptr, nullptr};  // the host loop's batches
+  // one of them, recorded behind the last launch of the frame's latest render;
+  // null if that was waited for.  What uses the counters or the scratch next
+  // waits for it on its stream.
+  cudaEvent_t tail = nullptr;
   // cached single-launch render graph and the launch parameters it was built for
   cudaGraphExec_t graph_exec = nullptr;
   cudaStream_t capture_stream = nullptr;   // private stream used only to record the graph

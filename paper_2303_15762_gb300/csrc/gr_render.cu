@@ -2401,6 +2401,15 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     *plan_bytes = total;
     return GR_OK;
   }
+  // the launches that the frame's last render left, maybe on another stream
+  if (f->tail) {
+    const cudaError_t ew = cudaStreamWaitEvent(st, f->tail, 0);
+    if (ew != cudaSuccess) {
+      err = std::string("stream wait: ") + cudaGetErrorString(ew);
+      return GR_E_CUDA;
+    }
+    f->tail = nullptr;
+  }
   if (f->scratch_bytes < total) {
     if (f->scratch) cudaFreeAsync(f->scratch, st);
     f->scratch = nullptr;
@@ -2483,9 +2492,9 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       return GR_E_CUDA;                          \
     }                                            \
   } while (0)
-  // From here on every exit waits for the stream: the next call on this frame,
-  // on whatever stream, resets the counters and the slots that this call's
-  // launches read, and may free its scratch.
+  // From here on an exit with launches in flight waits for them or leaves
+  // f->tail: the next call on this frame resets the counters and slots that
+  // they read.
   GR_CK(cudaMemcpyAsync(base + o_views, plan.views.data(), sizeof(DevView) * n_views, cudaMemcpyHostToDevice, st));
   GR_CK(cudaMemcpyAsync(base + o_vdesc, vd, sizeof(gr_view_desc) * n_views, cudaMemcpyHostToDevice, st));
   k_views<<<(n_views + 63) / 64, 64, 0, st>>>((const gr_view_desc*)(base + o_vdesc), (DevView*)(base + o_views), n_views);
@@ -2609,8 +2618,9 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
 
   // ---- iteration loop: batches of B iterations; the host watches the
   // device's live-slot count of the batch before the last one, so up to 2 B - 1
-  // iterations run past the end, ~13 us each, and the call returns when they
-  // are done.  At B = 8 / 4 / 2: 5.77 / 5.50 /
+  // iterations run past the end, ~13 us each; the last two, which find nothing
+  // to do, are left to f->tail (waiting for them: 5.28 -> 5.40 and 2.43 -> 2.51
+  // ms with the calls around the render).  At B = 8 / 4 / 2: 5.77 / 5.50 /
   // 5.41 ms (317 x 211 x 64 spp, anisotropic), 1.86 / 1.72 / 1.60 ms (256 x 192
   // x 16 spp); two iterations are still more device time than their launches
   // and the wait take on the host.
@@ -2691,9 +2701,9 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     }
     return GR_OK;
   }
-  cudaEvent_t ev[2];
-  cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming);
-  cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming);
+  cudaEvent_t* ev = f->ev;
+  for (int i = 0; i < 2; ++i)
+    if (!ev[i]) GR_CK(cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming));
   Counters* hc = f->ctr_host;
   long long it = 0;
   int batch = 0;
@@ -2710,6 +2720,7 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     // copy the counters of this batch into pinned slot (batch & 1)
     e = cudaMemcpyAsync(hc + (batch & 1), f->ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaEventRecord(ev[batch & 1], st);
+    f->tail = e == cudaSuccess ? ev[batch & 1] : nullptr;
     if (e != cudaSuccess) {
       err = std::string("counter copy: ") + cudaGetErrorString(e);
       status = GR_E_CUDA;
@@ -2738,10 +2749,10 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       break;
     }
   }
-  e = cudaStreamSynchronize(st);  // the last batch and its counter copy
-  if (e != cudaSuccess && status == GR_OK) {
-    err = std::string("render: ") + cudaGetErrorString(e);
-    status = GR_E_CUDA;
+  // an unfinished render's launches still add samples
+  if (status != GR_OK) {
+    cudaStreamSynchronize(st);
+    f->tail = nullptr;
   }
   f->iterations += it;
   if (profile) {
@@ -2750,6 +2761,7 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
       f->kernel_ms[k] = 0.0;
       f->kernel_launches[k] = 0;
     }
+    if (status == GR_OK && !pev.empty()) cudaEventSynchronize(pev.back());
     // launch order regen, trace, shadow, shade; reported as 0 regen, 1 trace,
     // 2 shade, 3 shadow
     const int slot_of[4] = {0, 1, 3, 2};
@@ -2764,8 +2776,6 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     }
     for (auto e3 : pev) cudaEventDestroy(e3);
   }
-  cudaEventDestroy(ev[0]);
-  cudaEventDestroy(ev[1]);
   return status;
 #undef GR_CK
 }
