@@ -1257,11 +1257,17 @@ __device__ __noinline__ int poisson_pick_fp64(double lam_d, float sigma_h_um, fl
   const double kd = 2.0 * kPiD / lam_d;
   double gd = 2.0 * kd * (double)sigma_h_um * (double)cos_i;
   gd *= gd;
-  double pd = exp(-gd), cd = pd;
+  double pd = exp(-gd), cd = pd, ratio = gd;
   int mi = 0;
-  while ((double)u >= cd && mi < 1000) {
+  // the next term's ratio g / m is formed beside the term and the sum, and the
+  // comparison is of the bits (neither is negative): an FP64 one takes a turn
+  // on the pipe that the chain waits for
+  const unsigned long long ub = (unsigned long long)__double_as_longlong((double)u);
+  while (ub >= (unsigned long long)__double_as_longlong(cd) && mi < 1000) {
     ++mi;
-    pd *= mi < 128 ? quotient(gd, (double)mi, c_rcp.r[mi]) : gd / mi;
+    pd *= ratio;
+    const double m = (double)(mi + 1);
+    ratio = mi < 127 ? quotient(gd, m, c_rcp.r[mi + 1]) : gd / m;
     cd += pd;
   }
   return mi;
