@@ -385,10 +385,11 @@ gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene
   const size_t o_eom = take(sizeof(int) * emitter_of_mat.size());
   const size_t o_etri = take(sizeof(float4) * etris.size());
   const size_t o_keys = take(sizeof(unsigned long long) * (size_t)n);
-  const size_t o_wide = take(sizeof(uint4) * 4 * (size_t)std::max(n - 1, 1));
+  const size_t wide_max = (size_t)gr::max_wide_nodes(n);
+  const size_t o_wide = take(sizeof(uint4) * 4 * wide_max);
   gr::GridDesc grid = {};
   bool grid_ok = false;
-  const size_t o_grid = take(sizeof(uint4) * 4 * (size_t)std::max(n - 1, 0));
+  const size_t o_grid = take(sizeof(uint4) * 4 * wide_max);
   int n_wide = 0;
   cudaError_t e = gr::dev_alloc(&S->mem, off, st);
   if (e != cudaSuccess) {

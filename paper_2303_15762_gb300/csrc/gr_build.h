@@ -23,6 +23,10 @@ cudaError_t dev_alloc(T** p, size_t bytes, cudaStream_t st) {
 struct GridDesc {
   float lo[3], step[3];
 };
+// Most 4-wide nodes the collapse of a tree of n triangles makes: a node has
+// four children, or only two or three leaves.  With a, b and c nodes of each
+// kind 3 a + b + 2 c = n - 1 and 2 b + 3 c <= n, so a + b + c <= (2 n - 1) / 3.
+inline int max_wide_nodes(int n) { return n < 2 ? 0 : (int)((2LL * n - 1) / 3); }
 cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* tri, int* tmat, float* nodes,
                         unsigned long long* keys_out, uint4* wn, uint4* gn, GridDesc* grid, bool* grid_ok,
                         int* n_wide, cudaStream_t st);

@@ -731,8 +731,8 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
 
 // Build the trees of `n` triangles (device arrays verts [n][9], tri_mat [n]).
 // Outputs (device, caller-allocated): tri [n][3] float4, tmat [n], nodes
-// [(n-1)][16] floats, keys [n], and the 4-wide nodes wn and gn of up to n - 1
-// nodes each; on the host *n_wide (their count, 0 if n < 2 or the tree is too
+// [(n-1)][16] floats, keys [n], and the 4-wide nodes wn and gn of up to
+// max_wide_nodes(n) each; on the host *n_wide (their count, 0 if n < 2 or the tree is too
 // deep for them), *grid (the grid of gn's boxes) and *grid_ok (whether it
 // serves the scene).  One scratch allocation;
 // the host waits once, for the state the launches leave behind, and again only

@@ -67,14 +67,15 @@ class Request:
 
     def scene_bytes_bound(self):
         """Upper bound of gr_scene_bytes for this scene: per triangle its
-        vertices (48 B), material (4), binary nodes (64), 4-wide nodes (64 on
-        the 16-bit grid, 64 in 8 bits), Morton key (8) and, for emitters, a vertex copy (48); per
-        material 64 + 4 B and an emitter record (96); per light 32 B; 256 B of
-        alignment for each of the 13 arrays."""
+        vertices (48 B), material (4), binary nodes (64), Morton key (8) and, for
+        emitters, a vertex copy (48); for every three triangles two 4-wide nodes
+        on the 16-bit grid and two in 8 bits (64 each); per material 64 + 4 B and
+        an emitter record (96); per light 32 B; 256 B of alignment for each of
+        the 13 arrays."""
         n = len(self.scene["tri_mat"])
         m = len(self.scene["mats"])
         L = len(self.scene["lights"])
-        return n * (48 + 4 + 64 + 64 + 64 + 8 + 48) + m * (64 + 4 + 96) + L * 32 + 13 * 256 + 4096
+        return n * (48 + 4 + 64 + 8 + 48) + 2 * n // 3 * 128 + m * (64 + 4 + 96) + L * 32 + 13 * 256 + 4096
 
 
 class ProgressiveServer:
