@@ -157,11 +157,15 @@ def pack_views(views):
 
 def _pack_rows(rows, words, ints):
     """Rows of the generators as the C structs: the same words in the same
-    order, the first `ints` as integers, the reserved last two zero."""
+    order, the first `ints` as integers (modulo 2^32, as ctypes stores them),
+    the reserved last two zero."""
     rows = np.asarray(rows, dtype=np.float32).reshape(-1, words)
+    kinds = rows[:, :ints]
+    if not np.all(np.isfinite(kinds)):
+        raise ValueError("a material's or light's kind is not a number")
     out = np.zeros((max(1, len(rows)), words), dtype=np.float32)
     out[:len(rows), :words - 2] = rows[:, :words - 2]
-    out.view(np.int32)[:len(rows), :ints] = rows[:, :ints].astype(np.int32)
+    out.view(np.uint32)[:len(rows), :ints] = np.mod(np.trunc(kinds).astype(np.float64), 2.0 ** 32)
     return out, len(rows)
 
 
