@@ -1963,13 +1963,19 @@ __global__ void k_tables(const TableBuildRow* rows, int n_rows, const DevView* v
 }
 
 // ------------------------------------------------------------------ readback
-// The accumulators run [bin][pixel][stokes], the image [pixel][bin][stokes]: a
-// block transposes tiles of 32 pixels x 32 bins in shared memory, so that both
-// sides are contiguous 32-element rows (one element: a pixel and bin's 1 or 4
-// Stokes components).  Reading one row per bin and thread instead fetched a
-// 32-byte sector for each element: four images of 3.3M
-// pixels x 16 bins took 414 us with their calls, now 330, one of 512^2 x 32
-// bins x 4 components 205 -> 100 us.
+// The accumulators run [bin][pixel][stokes], the image [pixel][bin][stokes].
+// Both sides are read and written as contiguous rows of 32 elements (one
+// element: a pixel and bin's 1 or 4 Stokes components), through shared memory:
+// reading one row per bin and thread instead fetched a 32-byte sector for each
+// element (16.8M floats: ~136 us with the call, whatever the bins).  From
+// kTileBins bins on a block transposes tiles of 32 pixels x 32 bins; with fewer
+// its lanes would idle as the rows of bins are stored, so a block takes a run of
+// pixels instead, whose image is one contiguous range.  16.8M floats, 1
+// component, tiles against runs (us): 801 and 100 with 1 bin, 234 and 91 with 4,
+// 143 and 88 with 8, 106 and 86 with 16, 92 and 86 with 24, 89 and 98 with 31;
+// 4 components: 253 and 69, 94 and 67, 72 and 67, 69 and 72, 66 and 68, 68 and
+// 70.  Runs of 32 KB: 104 to 112 us with 1 component.
+constexpr int kTileBins = 28, kRunBytes = 16384;
 struct Stokes4 {  // 4-byte aligned, where an accumulator or image is not 16-byte aligned
   float x, y, z, w;
 };
@@ -1982,6 +1988,30 @@ __device__ __forceinline__ V mean_of(const V& s, const V& c, float i) {
   r.z = (s.z - c.z) * i;
   r.w = (s.w - c.w) * i;
   return r;
+}
+template <class V>
+__global__ void __launch_bounds__(256) k_readback_run(const V* __restrict__ sum, const V* __restrict__ comp, int n_pix,
+                                                      int nb, int run, const float* __restrict__ inv_count,
+                                                      V* __restrict__ out) {
+  // run x nb <= kRun elements, one unused after each 128 bytes: lanes that
+  // store a bin of 32 neighbouring pixels meet different banks
+  constexpr int kRun = kRunBytes / (int)sizeof(V), kRow = 128 / (int)sizeof(V);
+  __shared__ V s[kRun + kRun / kRow];
+  const int pix0 = blockIdx.x * run, have = min(run, n_pix - pix0), lane = threadIdx.x & 31, rows = run / 32;
+#pragma unroll 4
+  for (int g = threadIdx.x >> 5; g < rows * nb; g += 8) {
+    const int b = g / rows, at = (g - b * rows) * 32 + lane;
+    if (at < have) {
+      const size_t a = (size_t)b * n_pix + pix0 + at;
+      const int e = at * nb + b;
+      s[e + e / kRow] = mean_of(sum[a], comp[a], inv_count[b]);
+    }
+  }
+  __syncthreads();
+  const int n = have * nb;
+  V* o = out + (size_t)pix0 * nb;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < n; e += 256) o[e] = s[e + e / kRow];
 }
 template <class V>
 __global__ void __launch_bounds__(256) k_readback(const V* __restrict__ sum, const V* __restrict__ comp, int n_pix,
@@ -3062,20 +3092,26 @@ gr_status render_static_impl(gr_scene* const* scenes, int n_scenes, const gr_vie
   return GR_OK;
 }
 
+template <class V>
+void launch_readback(const void* sum, const void* comp, int n_pix, int nb, const float* inv, void* out, cudaStream_t st) {
+  if (nb < kTileBins) {
+    const int run = kRunBytes / (int)sizeof(V) / nb / 32 * 32;
+    k_readback_run<V><<<((unsigned)n_pix + run - 1) / run, 256, 0, st>>>((const V*)sum, (const V*)comp, n_pix, nb, run, inv,
+                                                              (V*)out);
+  } else {
+    k_readback<V><<<dim3((n_pix + 31) / 32, (nb + 31) / 32), 256, 0, st>>>((const V*)sum, (const V*)comp, n_pix, nb, inv,
+                                                                          (V*)out);
+  }
+}
+
 cudaError_t readback_impl(gr_frame* f, int v, float* dst_dev, const float* inv_count_dev, cudaStream_t st) {
   const gr_view_shape& s = f->shapes[v];
   const float *sum = f->acc + f->offsets[v], *comp = f->acc + f->acc_floats + f->offsets[v];
   const int n_pix = s.W * s.H;
-  const dim3 grid((unsigned)((n_pix + 31) / 32), (unsigned)((s.nb + 31) / 32));
   const bool aligned = (((uintptr_t)sum | (uintptr_t)comp | (uintptr_t)dst_dev) & 15) == 0;
-  if (s.ns == 1)
-    k_readback<float><<<grid, 256, 0, st>>>(sum, comp, n_pix, s.nb, inv_count_dev, dst_dev);
-  else if (aligned)
-    k_readback<float4><<<grid, 256, 0, st>>>((const float4*)sum, (const float4*)comp, n_pix, s.nb, inv_count_dev,
-                                             (float4*)dst_dev);
-  else
-    k_readback<Stokes4><<<grid, 256, 0, st>>>((const Stokes4*)sum, (const Stokes4*)comp, n_pix, s.nb, inv_count_dev,
-                                              (Stokes4*)dst_dev);
+  if (s.ns == 1) launch_readback<float>(sum, comp, n_pix, s.nb, inv_count_dev, dst_dev, st);
+  else if (aligned) launch_readback<float4>(sum, comp, n_pix, s.nb, inv_count_dev, dst_dev, st);
+  else launch_readback<Stokes4>(sum, comp, n_pix, s.nb, inv_count_dev, dst_dev, st);
   return cudaGetLastError();
 }
 
