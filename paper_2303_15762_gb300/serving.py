@@ -206,7 +206,7 @@ class ProgressiveServer:
 
     def idle(self):
         with self._lock:
-            return not (self.waiting or self.ready or self.active)
+            return not (self.waiting or self._building or self.ready or self.active)
 
     def wait_prepared(self, timeout_s=60.0):
         """Block until the preparation thread has built every waiting request
