@@ -146,7 +146,7 @@ typedef struct {
  * into nodes of up to four children, with child boxes on a 16-bit grid over
  * the scene's bounds, rounded outward (64 bytes per node; a call with a scene
  * that has a coordinate beyond 1e12, a tree too deep, or more than one in 16 of whose triangles
- * is smaller than 8 steps of its grid, walks the FP32 nodes instead);
+ * is smaller than 2 steps of its grid, walks the FP32 nodes instead);
  * GR_FLAG_FP32_NODES walks the binary tree with FP32 child boxes (64 bytes per
  * node); GR_FLAG_WIDE_BVH traverses the 4-wide tree with 8-bit child boxes
  * relative to each node, one ray per thread (all three give the same closest

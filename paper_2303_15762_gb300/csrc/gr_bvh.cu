@@ -47,7 +47,7 @@ constexpr int kMaxLevels = 256;
 struct BuildState {
   int clo[3], chi[3];   // centroid bounds as ordered integers
   int lo[3], hi[3];     // vertex bounds as ordered integers
-  int bad, small;       // coordinates out of the grid's range; triangles smaller than 8 grid steps
+  int bad, small;       // coordinates out of the grid's range; triangles smaller than kSmallSteps grid steps
   int deep;             // a walk of the 4-wide grid nodes could need more than kGridStackDepth entries
   GridDesc g;
   int m[2], created[2]; // clusters left and nodes created, by parity of the round
@@ -559,10 +559,21 @@ __device__ __forceinline__ float half_area(const BoxF& b) {
 // The 16-bit grid of a scene: its bounds in 65535 steps per axis.  It serves
 // unless a coordinate is not finite or beyond 1e12, a walk of the tree could
 // need more than the kGridStackDepth entries it has, or it is so coarse against
-// the triangles (more than one in 16 smaller than 8 steps) that their boxes
-// would swell; the renders of such a scene walk the FP32 nodes.  The same
+// the triangles (more than one in 16 smaller than kSmallSteps steps) that their
+// boxes swell by more than the 4-wide walk saves; the renders of such a scene
+// walk the FP32 nodes.  k_trace of a 512^2 x 16 spp view of procedural objects
+// of 1 m on a ground that stretches the grid, grid nodes against FP32 nodes
+// (us): 83k triangles on 32 / 64 / 96 / 256 m 4165 / 5243 / 6747 / 11506
+// against 4637 / 5845 / 6385 / 7499; 7k on 128 / 256 m 4259 / 5254 against 4523
+// / 5086; 374k on 32 / 48 m 6312 / 8511 against 6769 / 8411; the first object
+// beside as many large triangles on 64 / 96 m 5506 / 6732 against 5702 / 6206.
+// In each of them the first ground where the grid loses is the first with
+// triangles smaller than 2 steps (11% to 24% of them).  Beyond the line the
+// binary FP16 nodes of before took 2 to 7% less than the FP32 nodes, and the
+// renders, with what surrounds the trace, no less.  The same
 // launch stores the box of every binary internal node (from its parent's
 // child boxes).
+constexpr float kSmallSteps = 2.0f;
 __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ tri, const float* __restrict__ nodes, int n,
                                                     BuildState* S, int parity, float* __restrict__ nbox,
                                                     int* __restrict__ front, int* __restrict__ pend) {
@@ -582,7 +593,7 @@ __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ t
   int small = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const BoxF b = leaf_box(tri, i);
-    small += fmaxf(fmaxf(b.hi[0] - b.lo[0], b.hi[1] - b.lo[1]), b.hi[2] - b.lo[2]) < 8.0f * widest;
+    small += fmaxf(fmaxf(b.hi[0] - b.lo[0], b.hi[1] - b.lo[1]), b.hi[2] - b.lo[2]) < kSmallSteps * widest;
     if (i >= n - 1) continue;
     const float4* q = (const float4*)(nodes + 16 * (size_t)i);
     const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
