@@ -208,12 +208,6 @@ __device__ __forceinline__ void start_sample(const RenderParams& p, int slot, in
   P.st8[slot] = ST_ACTIVE;
 }
 
-// Sum a per-thread count over the warp and add it with one atomic.
-__device__ __forceinline__ void warp_count(unsigned long long* ctr, int v) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0 && v) atomicAdd(ctr, (unsigned long long)v);
-}
-
 // Block-wide reservation of n entries per thread (n >= 0) with one atomic per
 // block: returns the first of this thread's n entries (exclusive scan over the
 // block).  Every thread of the block must call it (uniform control flow); the
@@ -627,11 +621,11 @@ constexpr int kGridLeaves = GR_GRID_LEAVES;
 // of 4 warps per issue) beside 58% busy ALUs at 17 of 32 lanes.  The 4-wide
 // grid nodes halve the chain: 13.2 visits per ray instead of 26.0, and 20%
 // fewer instructions; k_trace on 129M rays of a 512^2 x 256 spp render of 91k
-// triangles went from 38.6 to 31.7 ms (binary nodes with FP16 boxes before;
-// the same binary nodes on the grid: 37.8).  kGridLeaves 4 / 5 / 8: 34.4 /
-// 33.6 / 33.6 ms against 32.9 at 6; 2 / 3 / 4 visits between two looks at the
-// schedule: 35.4 / 34.0 / 32.9 ms against 32.5 at 6; 6 or 8 blocks per SM:
-// 34.3 / 37.1 ms against 34.0 at 7.
+// triangles went from 38.6 to 31.8 ms (binary nodes with FP16 boxes before;
+// the same binary nodes on the grid: 37.8).  Against those 31.8 ms: kGridLeaves
+// 4 / 5 / 8 33.8 / 32.6 / 32.4 instead of 6; 2 / 3 / 4 / 8 visits between two
+// looks at the schedule 34.0 / 32.5 / 32.2 / 32.5 instead of 6; 6 or 8 blocks
+// per SM 33.0 / 34.3 instead of 7.
 //   entry(e) -> slot of queue entry e; ray(slot, o, d, exclude) gives the
 //   ray and returns its scene; done(slot, hit) consumes a finished ray.
 template <int TREE, class Entry, class Ray, class Done>
