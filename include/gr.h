@@ -243,8 +243,9 @@ typedef struct {
 gr_status gr_scene_create(const gr_scene_desc* desc, void* cuda_stream, gr_scene** out);
 /* Free the scene.  Synchronises its device (another thread's render may still
  * read it).  The
- * library keeps up to 256 MB of freed device memory for its next calls (512 MB
- * while scenes or frames live) and gives it back when an allocation fails. */
+ * library keeps freed device memory for its next calls while it holds at most
+ * 512 MB in all (256 MB once no scene or frame lives) and gives it back when an
+ * allocation fails. */
 gr_status gr_scene_destroy(gr_scene* scene);
 /* Device bytes the scene holds (triangles, BVH layouts, materials, lights,
  * emitters); host-side bookkeeping, no CUDA call.  Errors: GR_E_INVALID. */

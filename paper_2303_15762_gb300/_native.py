@@ -159,14 +159,19 @@ def _pack_rows(rows, words, ints):
     """Rows of the generators as the C structs: the same words in the same
     order, the first `ints` as integers (modulo 2^32, as ctypes stores them),
     the reserved last two zero."""
-    rows = np.asarray(rows, dtype=np.float32).reshape(-1, words)
-    kinds = rows[:, :ints]
-    if not np.all(np.isfinite(kinds)):
-        raise ValueError("a material's or light's kind is not a number")
-    out = np.zeros((max(1, len(rows)), words), dtype=np.float32)
-    out[:len(rows), :words - 2] = rows[:, :words - 2]
-    out.view(np.uint32)[:len(rows), :ints] = np.mod(np.trunc(kinds).astype(np.float64), 2.0 ** 32)
-    return out, len(rows)
+    out = np.array(rows, dtype=np.float32).reshape(-1, words)
+    n = len(out)
+    if n == 0:
+        return np.zeros((1, words), dtype=np.float32), 0
+    kinds = out[:, :ints]
+    # int() refuses what is no number; a few rows are faster one by one
+    if n < 5 or not abs(kinds).max() < 2.0 ** 31:
+        kinds = [[(int(x) + 2 ** 31) % 2 ** 32 - 2 ** 31 for x in r] for r in kinds.tolist()]
+    else:
+        kinds = kinds.astype(np.int32)
+    out.view(np.int32)[:, :ints] = kinds
+    out[:, words - 2:] = 0.0
+    return out, n
 
 
 class Scene:

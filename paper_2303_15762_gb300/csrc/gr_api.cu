@@ -29,10 +29,12 @@ namespace gr {
 // One memory pool per device, created at its first use.  A pool that gives its
 // memory back at every synchronisation (the default one) makes each call map
 // and unmap it again: ~90 us per allocation of a few KB, 1 ms for 500 MB.  This
-// one keeps up to kPoolKeep bytes while scenes or frames live, and at most
-// kPoolIdle once the last of them is gone; what it keeps is given back when an
-// allocation of the library fails.  Allocation and release are stream-ordered
-// and safe from several threads.
+// one keeps what was freed while it holds at most kPoolKeep bytes in all, live
+// ones included; holding more (frames and scratch of large views), it gives
+// freed memory back at the next synchronisation as the default pool does.  Once
+// the last scene and frame is gone it keeps at most kPoolIdle; what it keeps is
+// given back when an allocation of the library fails.  Allocation and release
+// are stream-ordered and safe from several threads.
 namespace {
 constexpr size_t kPoolKeep = 512u << 20, kPoolIdle = 256u << 20;
 struct LibPool {
