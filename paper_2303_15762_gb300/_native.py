@@ -165,7 +165,7 @@ def _pack_rows(rows, words, ints):
         return np.zeros((1, words), dtype=np.float32), 0
     kinds = out[:, :ints]
     # int() refuses what is no number; a few rows are faster one by one
-    if n < 5 or not abs(kinds).max() < 2.0 ** 31:
+    if n < 5 or not abs(kinds.sum()) < 2.0 ** 31:
         kinds = [[(int(x) + 2 ** 31) % 2 ** 32 - 2 ** 31 for x in r] for r in kinds.tolist()]
     else:
         kinds = kinds.astype(np.int32)

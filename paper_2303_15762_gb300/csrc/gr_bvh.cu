@@ -576,7 +576,7 @@ __device__ __forceinline__ float half_area(const BoxF& b) {
 constexpr float kSmallSteps = 2.0f;
 __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ tri, const float* __restrict__ nodes, int n,
                                                     BuildState* S, int parity, float* __restrict__ nbox,
-                                                    int* __restrict__ front, int* __restrict__ pend) {
+                                                    int2* __restrict__ front) {
   if (S->m[parity] != 1) return;  // the clustering needs more rounds
   GridDesc g;
   float widest = 0.0f;
@@ -587,8 +587,7 @@ __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ t
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     S->g = g;
-    front[0] = 0;  // wide node 0 stands for the root
-    pend[0] = 0;
+    front[0] = make_int2(0, 0);  // wide node 0 stands for the root
   }
   int small = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -614,14 +613,15 @@ __global__ void __launch_bounds__(256) k_grid_steps(const float4* __restrict__ t
 }
 
 // One level of the top-down collapse.  front[w] is the binary node that wide
-// node w stands for, pend[w] the most entries a walk that enters w can have on
-// its stack: every node on the way pushed its internal children but the one
-// walked next.  (A bound by levels would not do: the way to w may have taken a
-// wide level for each binary one, with three entries left at each.)  Level L's nodes are [level_first[L], + level_count[L]),
-// and a node's internal children take consecutive places in the next level.
+// node w stands for, and the most entries a walk that enters w can have on its
+// stack: every node on the way pushed its internal children but the one walked
+// next.  (A bound by levels would not do: the way to w may have taken a wide
+// level for each binary one, with three entries left at each.)  Level L's nodes
+// are [level_first[L], + level_count[L]), and a node's internal children take
+// consecutive places in the next level.
 __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ nodes, const float* __restrict__ nbox,
-                                                  const float4* __restrict__ tri, int* __restrict__ front,
-                                                  int* __restrict__ pend, BuildState* S, int parity, int level, uint4* __restrict__ wn,
+                                                  const float4* __restrict__ tri, int2* __restrict__ front,
+                                                  BuildState* S, int parity, int level, uint4* __restrict__ wn,
                                                   uint4* __restrict__ gn) {
   if (S->m[parity] != 1) return;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -629,7 +629,8 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
   if (t == 0) S->level_first[level + 1] = first + count;
   if (t >= count) return;
   const GridDesc g = S->g;
-  const int widx = first + t, bnode = front[widx];
+  const int widx = first + t, bnode = front[widx].x;
+  int below = front[widx].y;
   int ch[4];
   int cnt = 2;
   ch[0] = __float_as_int(nodes[16 * bnode + 12]);
@@ -687,7 +688,7 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
   int refs[4] = {-1, -1, -1, -1};
   int inner = 0;
   for (int c = 0; c < cnt; ++c) inner += ch[c] >= 0;
-  const int below = pend[widx] + max(inner - 1, 0);
+  below += max(inner - 1, 0);
   if (below > kGridStackDepth) S->deep = 1;
   int w = inner ? first + count + atomicAdd(&S->level_count[level + 1], inner) : 0;
   for (int c = 0; c < cnt; ++c) {
@@ -695,8 +696,7 @@ __global__ void __launch_bounds__(128) k_collapse(const float* __restrict__ node
       refs[c] = ch[c];
     } else {
       refs[c] = w;
-      pend[w] = below;
-      front[w++] = ch[c];
+      front[w++] = make_int2(ch[c], below);
     }
   }
   uint4 a, b, c4, d;
@@ -805,15 +805,15 @@ cudaError_t build_trees(const float* verts, const int* tri_mat, int n, float4* t
       k_ploc_tail<<<1, kTail, 0, st>>>(Bc, Cc, S, parity, n, nodes);
       // the collapse is enqueued with the rounds; its launches return at once
       // if the clustering is not done, and are enqueued again after the next ones
-      float* nbox = Bc;  // the cluster boxes, ids and pairs have served
-      int *front = Cc, *pend = P;
-      k_grid_steps<<<std::min(g256, 1024), 256, 0, st>>>(tri, nodes, n, S, parity, nbox, front, pend);
+      float* nbox = Bc;  // the cluster boxes and ids have served
+      int2* front = (int2*)(d + o_id);  // 2 n ints for at most (2 n - 1) / 3 of them
+      k_grid_steps<<<std::min(g256, 1024), 256, 0, st>>>(tri, nodes, n, S, parity, nbox, front);
       int level = 0, batch = first_levels(n);
       do {
         for (int k = 0; k < batch && level < kMaxLevels; ++k, ++level) {
           const double widest = level < 14 ? std::pow(4.0, level) : 3e8;
           const int blocks = (int)((std::min(widest, (double)n) + 127) / 128);
-          k_collapse<<<blocks, 128, 0, st>>>(nodes, nbox, tri, front, pend, S, parity, level, wn, gn);
+          k_collapse<<<blocks, 128, 0, st>>>(nodes, nbox, tri, front, S, parity, level, wn, gn);
         }
         batch = kMoreLevels;
         if ((r = cudaMemcpyAsync(&h, S, sizeof h, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return r;

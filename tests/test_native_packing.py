@@ -16,13 +16,14 @@ def _material(**words):
 
 
 @pytest.mark.parametrize("words", [{}, dict(w0=3.9), dict(w1=-0.9), dict(w0=-2.0), dict(w0=3e9), dict(w1=2.0 ** 40), dict(w0=-1e38)])
-def test_struct_fields(words):
-    out, n = nat._pack_rows([_material(), _material(**words)], 16, 2)
+@pytest.mark.parametrize("rows", [2, 70])
+def test_struct_fields(words, rows):
+    out, n = nat._pack_rows([_material()] * (rows - 1) + [_material(**words)], 16, 2)
     r = _material(**words)
-    m = nat.gr_material.from_buffer_copy(out[1].tobytes())
+    m = nat.gr_material.from_buffer_copy(out[-1].tobytes())
     want = nat.gr_material()
     want.type, want.fresnel = int(r[0]), int(r[1])
-    assert n == 2 and (m.type, m.fresnel) == (want.type, want.fresnel)
+    assert n == rows and (m.type, m.fresnel) == (want.type, want.fresnel)
     assert [m.n_re, m.n_im, m.period_um, m.height_um, *m.gdir] == [float(x) for x in r[2:9]]
     assert [m.sigma_h_um, m.corr_len_um, m.Le, m.coh_len_um, m.cauchy_b_um2] == [float(x) for x in r[9:14]]
     assert not np.any(out[:, 14:])
@@ -30,9 +31,10 @@ def test_struct_fields(words):
 
 @pytest.mark.parametrize("word", [0, 1])
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
-def test_kind_that_is_no_number(word, value):
+@pytest.mark.parametrize("rows", [1, 70])
+def test_kind_that_is_no_number(word, value, rows):
     with pytest.raises((ValueError, OverflowError)):
-        nat._pack_rows([_material(**{"w%d" % word: value})], 16, 2)
+        nat._pack_rows([_material()] * (rows - 1) + [_material(**{"w%d" % word: value})], 16, 2)
 
 
 def test_lights():
