@@ -2649,8 +2649,8 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
   // ---- iteration loop: batches of B iterations; the host watches the
   // device's live-slot count of the batch before the last one, so up to 2 B - 1
   // iterations run past the end, ~13 us each; the last two, which find nothing
-  // to do, are left to f->tail (waiting for them: 5.28 -> 5.40 and 2.43 -> 2.51
-  // ms with the calls around the render).  At B = 8 / 4 / 2: 5.77 / 5.50 /
+  // to do, are left to f->tail (a 256 x 192 preview's call that waits for them:
+  // 2.45 -> 2.51 ms).  At B = 8 / 4 / 2: 5.77 / 5.50 /
   // 5.41 ms (317 x 211 x 64 spp, anisotropic), 1.86 / 1.72 / 1.60 ms (256 x 192
   // x 16 spp); two iterations are still more device time than their launches
   // and the wait take on the host.
