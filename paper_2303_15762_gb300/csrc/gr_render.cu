@@ -1227,23 +1227,24 @@ __device__ __noinline__ int grating_pick_fp64(double lam_d, float height_um, int
   return 0x7fffffff;
 }
 
-// 1 / m for m < 128 (the term counts of g <= kGCont).
+// 1 / m for m < 128 (the term counts of g <= kGCont) as the nearest FP64 value
+// and what it leaves: 1 - m hi is formed exactly from hi's leading 24 bits and
+// the rest.
 struct RcpTable {
-  double r[128];
-  constexpr RcpTable() : r() {
-    for (int m = 1; m < 128; ++m) r[m] = 1.0 / m;
+  double hi[128], lo[128];
+  constexpr RcpTable() : hi(), lo() {
+    for (int m = 1; m < 128; ++m) {
+      hi[m] = 1.0 / m;
+      const double lead = (double)(float)hi[m];
+      lo[m] = ((1.0 - m * lead) - m * (hi[m] - lead)) / m;
+    }
   }
 };
 __constant__ RcpTable c_rcp = RcpTable();
-
-// g / m from the rounded reciprocal r of m: the product corrected by its exact
-// remainder is the correctly rounded quotient (Markstein, "Computation of
-// elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
-// Dev. 1990), in three operations beside the serial product of the terms.
-__device__ __forceinline__ double quotient(double g, double m, double r) {
-  const double q = g * r;
-  return fma(fma(-q, m, g), r, q);
-}
+// g / m, correctly rounded: a quotient by m < 128 that is not an FP64 value lies
+// at least 1 / (2 m) of a unit in the last place from the middle between two,
+// far more than what the two operations leave out.
+__device__ __forceinline__ double quotient(double g, int m) { return fma(g, c_rcp.hi[m], g * c_rcp.lo[m]); }
 
 // Rough-surface term count m ~ Poisson(g), g = (2 k sigma_h cos_i)^2: the
 // first m whose cumulative Poisson probability exceeds u (at most 1000).
@@ -1260,8 +1261,7 @@ __device__ __noinline__ int poisson_pick_fp64(double lam_d, float sigma_h_um, fl
   while (ub >= (unsigned long long)__double_as_longlong(cd) && mi < 1000) {
     ++mi;
     pd *= ratio;
-    const double m = (double)(mi + 1);
-    ratio = mi < 127 ? quotient(gd, m, c_rcp.r[mi + 1]) : gd / m;
+    ratio = mi < 127 ? quotient(gd, mi + 1) : gd / (mi + 1);
     cd += pd;
   }
   return mi;
