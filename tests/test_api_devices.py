@@ -63,8 +63,9 @@ def api(tmp_path_factory):
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     subprocess.check_call([nvcc] + gb.ARCH + gb.NVCC_FLAGS + ["-c", os.path.join(gb.CSRC, "gr_api.cu"),
                                                               "-o", str(d / "api.o")])
-    # the kernels' translation units are left out: the entry points under test call none of them
-    subprocess.check_call(["g++", "-std=c++17", "-fPIC", "-shared", "-I", cuda, "-o", str(d / "api.so"),
+    # (its own runtime, also where a process has the real one; the kernels' translation units
+    # are left out: the entry points under test call none of them)
+    subprocess.check_call(["g++", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", cuda, "-o", str(d / "api.so"),
                            str(d / "runtime.cpp"), str(d / "api.o")])
     L = ctypes.CDLL(str(d / "api.so"), mode=os.RTLD_LAZY)
     L.fake_log.restype = ctypes.c_char_p
