@@ -54,13 +54,13 @@ FLOP_PER_GNODE = 79
 KERNELS = ["k_regen", "k_trace", "k_shade", "k_shadow"]
 # DRAM traffic of the dominant kernel per unit (ray) from one ncu capture:
 # dram__bytes_read.sum + dram__bytes_write.sum of the second k_trace launch of
-# the 256x256 x 64 spp case (164.61 + 8.28 MB), divided by the rays it traced
+# the 256x256 x 64 spp case (164.44 + 8.08 MB), divided by the rays it traced
 # (the full default pool: one slot per ticket, 2,097,152 slots, all live in
 # the second iteration, plus about a thousand next-event rays, not counted);
 # traffic grows with the rays a launch processes.  Valid only for the
 # traversal sources whose hash (source_hash) is recorded with it (else
 # reported null).
-NCU_TRAFFIC_PER_RAY = {("k_trace", "8c7e888533247cf0"): (164.607232e6 + 8.280320e6) / 2097152}
+NCU_TRAFFIC_PER_RAY = {("k_trace", "447721aee4ddb35e"): (164.436992e6 + 8.076800e6) / 2097152}
 # the glass workload: a constant environment of this radiance lets paths
 # refracted through the glass reach a light, and the oracle crop (x0, y0,
 # side) is where the glass decides the most pixel-bins of the 512^2 view

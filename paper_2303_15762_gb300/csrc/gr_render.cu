@@ -618,7 +618,7 @@ constexpr int kGridLeaves = GR_GRID_LEAVES;
 // least (t, id) over the triangles whose boxes the ray enters, whatever the
 // tree and the schedule; only the counts of visits and tests differ.
 // What bounds it: the chain of dependent node fetches (long-scoreboard stalls
-// of 4 warps per issue) beside 58% busy ALUs at 17 of 32 lanes.  The 4-wide
+// of 4 warps per issue) beside 57% busy ALUs at 16 of 32 lanes.  The 4-wide
 // grid nodes halve the chain: 13.2 visits per ray instead of 26.0, and 20%
 // fewer instructions; k_trace on 129M rays of a 512^2 x 256 spp render of 91k
 // triangles went from 38.6 to 31.8 ms (binary nodes with FP16 boxes before;
