@@ -76,22 +76,25 @@ void count_object(int dev, int change) {
 }
 }  // namespace
 
+// A failure is returned and not left behind for the next call's cudaGetLastError.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
   const cudaMemPool_t pool = pool_of(dev);
-  if (!pool) return cudaMallocAsync(p, bytes, st);
-  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
   if (e == cudaSuccess) return e;
   cudaGetLastError();
+  if (!pool) return e;
   if (e == cudaErrorMemoryAllocation) {
     // what the pool keeps may be in the way, in pieces too small
     cudaStreamSynchronize(st);
     cudaMemPoolTrimTo(pool, 0);
-    cudaGetLastError();
-    return cudaMallocFromPoolAsync(p, bytes, pool, st);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  } else {
+    e = cudaMallocAsync(p, bytes, st);  // the pool is gone (its device was reset)
   }
-  return cudaMallocAsync(p, bytes, st);  // the pool is gone (its device was reset)
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 // Pinned counters of a frame (two Counters): pairs of one 64-pair block, kept

@@ -2445,6 +2445,8 @@ gr_status render_impl(gr_scene* const* scenes, int n_scenes, const gr_view_desc*
     f->scratch = nullptr;
     f->scratch_bytes = 0;
     if (dev_alloc(&f->scratch, total, st) != cudaSuccess) {
+      f->scratch = nullptr;
+      cudaStreamSynchronize(st);  // behind what was f->tail
       err = "scratch allocation failed";
       return GR_E_OOM;
     }

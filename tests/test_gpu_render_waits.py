@@ -56,3 +56,22 @@ def test_next_use_comes_after(gr, pool):
         f.reset(stream=_handle(x))
         gr.render([s], [v], f, stream=_handle(x), **opts)
         assert np.array_equal(f.readback(0, stream=_handle(y)), image)
+
+
+def test_failed_allocation_leaves_nothing_running(gr):
+    import torch
+    s = gr.Scene(sg.procedural_scene(seed=4, n_objects=4, target_tris=3000))
+    v = sg.procedural_view(width=640, height=480, n_bins=8, n_stokes=1, spp=8)
+    many = dict(sg.procedural_view(width=8192, height=8192, n_bins=16, n_stokes=1, spp=16), view_index=0)
+    f, g = gr.Frame([v]), gr.Frame([many])
+    torch.cuda.synchronize()
+    x, y = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(3):
+        gr.render([s], [v], f, stream=_handle(x), seed=2, flags=gr.FLAG_NEE)
+        want = f.readback(0, stream=_handle(x))
+        # frames[0]'s scratch serves the call: 2^30 slots of 429 bytes, more than any device has
+        with pytest.raises(gr.GrError, match="scratch allocation failed"):
+            gr.render_multi([s], [v, many], [f, g], [0, 0], stream=_handle(y), seed=2, flags=gr.FLAG_NEE | gr.FLAG_HERO,
+                            pool_size=(1 << 30) - 256)
+        assert x.query() and y.query()
+        assert np.array_equal(f.readback(0), want)
